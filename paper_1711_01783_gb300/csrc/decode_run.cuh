@@ -84,7 +84,6 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
     int sm_count = 152;
     cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, d->device);
     const dim3 syn_grid(syndrome_blocks(h.n_cn, sm_count), slabs);
-    const int cap_blocks = sm_count * 16;  // two waves of 8 blocks per SM
     // staged check updates: one wave of kStagedBlocksPerSm blocks per SM
     const int staged_cap = d->staging != MLD_STAGE_DIRECT ? sm_count * kStagedBlocksPerSm : 0;
     const int lane_blocks = (batch + 127) / 128;
@@ -145,8 +144,8 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
                 for (const mld::LayerLaunch &ll : g->layer_launches) {
                     const mld::CheckClass &k = h.classes[ll.cls];
                     la.cptr = g->leptr + ll.p0;
-                    const int blocks = std::max(1, std::min(grid_x(static_cast<int64_t>(ll.count) * TPC),
-                                                            sm_count * kLayeredBlocksPerSm));
+                    const int blocks = layer_blocks(grid_x(static_cast<int64_t>(ll.count) * TPC), k.dc < 0 ? -1 : k.dc + k.dd,
+                                                    sm_count);
                     ClassLaunch cl{k.c0, ll.count, k.dc, k.dc + k.dd, ll.e0, k.s0, blocks};
                     launch_layered<MsgT, W>(la, cl, g->lchk + ll.p0, slabs, s, hard1);
                 }
@@ -158,13 +157,13 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
                 }
             } else {
                 if (big < 0) {
-                    for (const ClassLaunch &cl : launches) launch_check_class<MsgT, W>(c2, cl, slabs, s, cap_blocks, hard1, staged_cap, d->staging);
+                    for (const ClassLaunch &cl : launches) launch_check_class<MsgT, W>(c2, cl, slabs, s, sm_count, hard1, staged_cap, d->staging);
                 } else {
                     MLD_CUDA(cudaEventRecord(d->ev_fork, s));
                     MLD_CUDA(cudaStreamWaitEvent(d->side, d->ev_fork, 0));
-                    launch_check_class<MsgT, W>(c2, launches[big], slabs, s, cap_blocks, hard1, staged_cap, d->staging);
+                    launch_check_class<MsgT, W>(c2, launches[big], slabs, s, sm_count, hard1, staged_cap, d->staging);
                     for (size_t i = 0; i < launches.size(); ++i)
-                        if (static_cast<int>(i) != big) launch_check_class<MsgT, W>(c2, launches[i], slabs, d->side, cap_blocks, hard1, staged_cap, d->staging);
+                        if (static_cast<int>(i) != big) launch_check_class<MsgT, W>(c2, launches[i], slabs, d->side, sm_count, hard1, staged_cap, d->staging);
                     MLD_CUDA(cudaEventRecord(d->ev_join, d->side));
                     MLD_CUDA(cudaStreamWaitEvent(s, d->ev_join, 0));
                 }
@@ -270,9 +269,8 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
                 for (const mld::LayerLaunch &ll : g->layer_launches) {
                     const mld::CheckClass &k = h.classes[ll.cls];
                     la.cptr = g->leptr + ll.p0;
-                    // one wave: the kernels loop over the launch's checks
-                    const int blocks = std::max(1, std::min(grid_x(static_cast<int64_t>(ll.count) * TPC),
-                                                            sm_count * kLayeredBlocksPerSm));
+                    const int blocks = layer_blocks(grid_x(static_cast<int64_t>(ll.count) * TPC), k.dc < 0 ? -1 : k.dc + k.dd,
+                                                    sm_count);
                     ClassLaunch cl{k.c0, ll.count, k.dc, k.dc + k.dd, ll.e0, k.s0, blocks};
                     launch_layered<MsgT, W>(la, cl, g->lchk + ll.p0, slabs, st, hard1);
                 }
@@ -313,7 +311,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
         {
             int s = timed_launch(d, kClsCheck, st, "k_check_update", [&] {
                 if (big < 0) {
-                    for (const ClassLaunch &cl : launches) launch_check_class<MsgT, W>(ca, cl, slabs, st, cap_blocks, hard1, staged_cap, d->staging);
+                    for (const ClassLaunch &cl : launches) launch_check_class<MsgT, W>(ca, cl, slabs, st, sm_count, hard1, staged_cap, d->staging);
                     return;
                 }
                 // the largest class on the caller's stream; the others on the
@@ -321,9 +319,9 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
                 // drains (errors of the event calls surface as the launch error)
                 cudaEventRecord(d->ev_fork, st);
                 cudaStreamWaitEvent(d->side, d->ev_fork, 0);
-                launch_check_class<MsgT, W>(ca, launches[big], slabs, st, cap_blocks, hard1, staged_cap, d->staging);
+                launch_check_class<MsgT, W>(ca, launches[big], slabs, st, sm_count, hard1, staged_cap, d->staging);
                 for (size_t i = 0; i < launches.size(); ++i)
-                    if (static_cast<int>(i) != big) launch_check_class<MsgT, W>(ca, launches[i], slabs, d->side, cap_blocks, hard1, staged_cap, d->staging);
+                    if (static_cast<int>(i) != big) launch_check_class<MsgT, W>(ca, launches[i], slabs, d->side, sm_count, hard1, staged_cap, d->staging);
                 cudaEventRecord(d->ev_join, d->side);
                 cudaStreamWaitEvent(st, d->ev_join, 0);
             }, static_cast<int>(launches.size()));

@@ -22,6 +22,7 @@ const char *last_error_text();
 namespace {
 
 constexpr int kK = 4;          // codewords per thread
+constexpr int kP = kK / 2;     // pairs of codewords per thread
 constexpr int kBlock = 128;
 
 // ---------------------------------------------------------------------------
@@ -124,19 +125,48 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
     return d;
 }
 
-// phi of four values with the result floored at `lo`, base-2 fits: the max
+// phi(|x|) of two values with the result floored at `lo`, base-2 fits: the max
 // of the two pieces and the floor in one instruction per value.  With
 // lo = phi(lmax) this equals phi of the argument clamped above at lmax (phi
 // decreases), and an argument of +inf gives lo (the small piece is -inf,
 // the large one 0), so the clamp needs no instruction of its own.
+// The polynomials run on packed pairs (two codewords per FMA-pipe
+// instruction, each half rounded as the scalar instruction rounds it; a
+// coefficient's sign moves, which changes no rounding).  lg2 and ex2 take |x|
+// as an operand modifier, so the magnitude is never formed; the subtraction
+// of lg2 stays scalar (packed it needs the two results as a register pair:
+// 0.285 against 0.299 ms, rate 0.1, n = 10^6, 64 codewords, half).
 template <int F>
-__device__ __forceinline__ float4 phi4_floor(float4 x, float lo) {
-    static_assert(F == kFitB2 || F == kFitB2H, "phi4_floor: base-2 fits only");
-    return make_float4(max3f(phi_small<F>(x.x), phi_large<F>(x.x), lo),
-                       max3f(phi_small<F>(x.y), phi_large<F>(x.y), lo),
-                       max3f(phi_small<F>(x.z), phi_large<F>(x.z), lo),
-                       max3f(phi_small<F>(x.w), phi_large<F>(x.w), lo));
+__device__ __forceinline__ float2 phi2_floor(float2 x, float lo) {
+    static_assert(F == kFitB2 || F == kFitB2H, "phi2_floor: base-2 fits only");
+    auto both = [](float v) { return make_float2(v, v); };
+    const float2 t = __fmul2_rn(x, x);
+    float2 ps;
+    if constexpr (F == kFitB2H) {
+        ps = __ffma2_rn(both(-MLD_PHI2H_S1), t, both(-MLD_PHI2H_S0));
+    } else {
+        ps = __ffma2_rn(both(-MLD_PHI2_S3), t, both(-MLD_PHI2_S2));
+        ps = __ffma2_rn(ps, t, both(-MLD_PHI2_S1));
+        ps = __ffma2_rn(ps, t, both(-MLD_PHI2_S0));
+    }
+    ps = __ffma2_rn(t, ps, both(MLD_PHI2_C0));
+    const float2 small = make_float2(ps.x - mufu_lg2(fabsf(x.x)), ps.y - mufu_lg2(fabsf(x.y)));
+    const float2 e = make_float2(mufu_ex2(-fabsf(x.x)), mufu_ex2(-fabsf(x.y)));
+    const float2 z = __fmul2_rn(e, e);
+    float2 pl;
+    if constexpr (F == kFitB2H) {
+        pl = __ffma2_rn(both(MLD_PHI2H_L1), z, both(MLD_PHI2H_L0));
+    } else {
+        pl = __ffma2_rn(both(MLD_PHI2_L3), z, both(MLD_PHI2_L2));
+        pl = __ffma2_rn(pl, z, both(MLD_PHI2_L1));
+        pl = __ffma2_rn(pl, z, both(MLD_PHI2_L0));
+    }
+    const float2 large = __fmul2_rn(e, pl);
+    return make_float2(max3f(small.x, large.x, lo), max3f(small.y, large.y, lo));
 }
+
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 
 template <typename T> struct IsHalf { static constexpr bool value = false; };
 template <> struct IsHalf<__half> { static constexpr bool value = true; };
@@ -147,11 +177,35 @@ __device__ __forceinline__ float clampf(float x, float lo, float hi) {
     return fminf(fmaxf(x, lo), hi);
 }
 
+__device__ __forceinline__ uint32_t fbits(float x) { return __float_as_uint(x); }
+__device__ __forceinline__ float bitsf(uint32_t x) { return __uint_as_float(x); }
+constexpr uint32_t kSign = 0x80000000u;
+
+// Sign word of a pair of codewords: the sign of a.x in bit 15, of a.y in bit
+// 31, as in a pair of halves (the other bits carry no meaning).  One byte
+// permutation for two codewords; words are XORed to form sign products.
+constexpr uint32_t kSignPair = 0x80008000u;
+__device__ __forceinline__ uint32_t sign_word(float2 a) { return __byte_perm(fbits(a.x), fbits(a.y), 0x7632); }
+// the sign of codeword k (0 or 1) of a sign word, as a float's sign bit
+__device__ __forceinline__ uint32_t sign_of(uint32_t w, int k) { return (k == 0 ? w << 16 : w) & kSign; }
+// the sign word of a pair whose codewords are negative where bits 0 and 1 are set
+__device__ __forceinline__ uint32_t sign_word_of_bits(uint32_t b) { return (b & 1u) << 15 | (b & 2u) << 30; }
+// non-negative values with the signs of two sign words
+__device__ __forceinline__ float4 with_signs(float2 m0, float2 m1, uint32_t w0, uint32_t w1) {
+    return make_float4(bitsf(fbits(m0.x) | sign_of(w0, 0)), bitsf(fbits(m0.y) | sign_of(w0, 1)),
+                       bitsf(fbits(m1.x) | sign_of(w1, 0)), bitsf(fbits(m1.y) | sign_of(w1, 1)));
+}
+
 // ---------------------------------------------------------------------------
 // 4-codeword vector access for each message storage type
 // ---------------------------------------------------------------------------
 template <typename T> struct Msg;
 template <> struct Msg<float> {
+    // four values as they are stored, and one pair of them as float
+    using Raw = float4;
+    static __device__ __forceinline__ float2 pair(const Raw &r, int p) {
+        return p == 0 ? make_float2(r.x, r.y) : make_float2(r.z, r.w);
+    }
     static __device__ __forceinline__ float4 load(const float *p) {
         return *reinterpret_cast<const float4 *>(p);
     }
@@ -163,8 +217,17 @@ template <> struct Msg<float> {
         *reinterpret_cast<float4 *>(p) = v;
         return v;
     }
+    // store the non-negative values of two pairs with the signs of two sign
+    // words (sign_word)
+    static __device__ __forceinline__ void store_signed(float *p, float2 m0, float2 m1, uint32_t w0, uint32_t w1) {
+        store(p, with_signs(m0, m1, w0, w1));
+    }
 };
 template <> struct Msg<__half> {
+    using Raw = uint2;
+    static __device__ __forceinline__ float2 pair(const Raw &r, int p) {
+        return __half22float2(*reinterpret_cast<const __half2 *>(p == 0 ? &r.x : &r.y));
+    }
     static __device__ __forceinline__ float4 load(const __half *p) {
         const uint2 u = *reinterpret_cast<const uint2 *>(p);
         const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&u.x));
@@ -188,6 +251,16 @@ template <> struct Msg<__half> {
         *reinterpret_cast<uint2 *>(p) = u;
         const float2 fa = __half22float2(a), fb = __half22float2(b);
         return make_float4(fa.x, fa.y, fb.x, fb.y);
+    }
+    // (rounding is symmetric, so the signs can go onto the rounded pair: one
+    // instruction for two codewords)
+    static __device__ __forceinline__ void store_signed(__half *p, float2 m0, float2 m1, uint32_t w0, uint32_t w1) {
+        const __half2 a = __floats2half2_rn(m0.x, m0.y);
+        const __half2 b = __floats2half2_rn(m1.x, m1.y);
+        uint2 u;
+        u.x = *reinterpret_cast<const uint32_t *>(&a) ^ (w0 & kSignPair);
+        u.y = *reinterpret_cast<const uint32_t *>(&b) ^ (w1 & kSignPair);
+        *reinterpret_cast<uint2 *>(p) = u;
     }
 };
 
@@ -307,15 +380,14 @@ __device__ __forceinline__ void emit_deg1_bits(const CnArgs &a, int slab, int sl
     if (valid && (lane0 & 7) == 0) *hb = static_cast<uint8_t>(nib | (other << 4));
 }
 
-// Message store under early termination: converged lanes keep their
-// messages frozen.  The freeze is not needed for exact outputs (a converged
-// codeword's posterior and decisions are frozen by the variable update and
-// emit_deg1*, and no output reads its later messages), so the
-// decisions-only kernels skip it (FREEZE false), which saves a reload and
-// four selects per term once lanes have converged.
-template <typename MsgT, int W, bool FREEZE = true>
+// Message store that keeps the messages of converged lanes.  The freeze is not
+// needed for exact outputs (a converged codeword's posterior and decisions
+// are frozen by the variable update and emit_deg1*, and no output reads its
+// later messages), so the decisions-only kernels store without it, which
+// saves a reload and four selects per term once lanes have converged.
+template <typename MsgT, int W>
 __device__ __forceinline__ void store_r(const CnArgs &a, MsgT *rp, float4 rv, uint32_t donenib) {
-    if (FREEZE && donenib) {
+    if (donenib) {
         const float4 old = Msg<MsgT>::load(rp);
         if (donenib & 1) rv.x = old.x;
         if (donenib & 2) rv.y = old.y;
@@ -327,147 +399,174 @@ __device__ __forceinline__ void store_r(const CnArgs &a, MsgT *rp, float4 rv, ui
 
 using mld::ClassLaunch;
 
-__device__ __forceinline__ uint32_t fbits(float x) { return __float_as_uint(x); }
-__device__ __forceinline__ float bitsf(uint32_t x) { return __uint_as_float(x); }
-constexpr uint32_t kSign = 0x80000000u;
+// What a check pass does beside the messages, at compile time, so that the
+// pass that runs most often carries no branch, load or register of the others.
+//   kPassPlain: messages only (an iteration of a fixed-iteration decode that
+//               is not its last);
+//   kPassFull:  a.final_pass and a.et are read: degree-1 posteriors and
+//               decisions, converged lanes frozen (last iterations, early
+//               termination with soft output, staged kernels);
+//   kPassHard:  early termination without soft output: a degree-1 VN gets its
+//               decision only, not its posterior.
+enum { kPassPlain = 0, kPassFull = 1, kPassHard = 2 };
 
-// Check j of one class (DC core edges and DD degree-1 VNs per check, all
-// terms in registers), codewords lane0 .. lane0+3 of the slab.  A thread past
-// the class end works on its last check and stores nothing (so a whole
-// shuffle pair stays active).  HARD1: a degree-1 VN gets its decision only,
-// not its posterior (early termination without soft output); FUSE (with
-// HARD1): with a.fuse the call also returns the previous iteration's
-// syndrome failures of the check for the thread's 4 codewords (bit k:
-// codeword lane0 + k), else 0.
-// Where a check's terms are read from.  TermsGlobal: straight from the
-// posterior, message and degree-1 arrays, the core VNs' column indices
-// loaded first; lv(i) / ro(i): posterior and stored message of core term i,
-// p1(i): phi term of degree-1 term i, each for the thread's 4 codewords.
-template <typename MsgT, int W, int DC>
-struct TermsGlobal {
-    const float *lvb;
-    const MsgT *rb;
-    const float *p1b;
-    int32_t e0, s0;
-    int32_t vidx[DC > 0 ? DC : 1];
-    __device__ __forceinline__ float4 lv(int i) const { return ldf4(lvb + static_cast<size_t>(vidx[i]) * W); }
-    __device__ __forceinline__ float4 ro(int i) const {
-        return Msg<MsgT>::load(rb + static_cast<size_t>(e0 + i) * W);
-    }
-    __device__ __forceinline__ float4 p1(int i) const { return ldf4(p1b + static_cast<size_t>(s0 + i) * W); }
-};
-
-template <typename MsgT, int W, int DC, int DD, bool HARD1, bool ACC, bool FUSE, typename Terms>
-__device__ __forceinline__ uint32_t check_terms(const CnArgs &a, int lane0, int slab, bool valid, int32_t e0,
-                                                int32_t s0, uint32_t sb, uint32_t donenib, const Terms &t);
-
-template <typename MsgT, int W, int DC, int DD, bool HARD1 = false, bool ACC = false, bool FUSE = HARD1>
-__device__ __forceinline__ uint32_t check_regular(const CnArgs &a, const ClassLaunch &cl, int32_t j, int lane0,
-                                                  int slab) {
-    constexpr int NB = W / 8;
-    const int32_t count = cl.count;
-    const bool valid = j < count;
-    if (!valid) j = count - 1;
-    const int32_t c = cl.c0 + j;
-    const int32_t e0 = cl.e0 + j * DC;
-    const int32_t s0 = cl.s0 + j * DD;
-
-    const uint32_t sb =
-        (static_cast<uint32_t>(a.sbits[(static_cast<size_t>(slab) * a.n_cn + c) * NB + lane0 / 8]) >>
-         (lane0 & 7));
-    const uint32_t donenib = a.et ? done_nibble<W>(a.done, slab, lane0) : 0u;
-    TermsGlobal<MsgT, W, DC> t;
-    t.rb = static_cast<const MsgT *>(a.r) + static_cast<size_t>(slab) * a.e_core * W + lane0;
-    t.lvb = a.Lv + static_cast<size_t>(slab) * a.n_core * W + lane0;
-    t.p1b = a.phi1 + static_cast<size_t>(slab) * a.n_deg1 * W + lane0;
-    t.e0 = e0;
-    t.s0 = s0;
-#pragma unroll
-    for (int i = 0; i < DC; ++i) t.vidx[i] = __ldg(a.col + e0 + i);
-    return check_terms<MsgT, W, DC, DD, HARD1, ACC, FUSE>(a, lane0, slab, valid, e0, s0, sb, donenib, t);
+// ---------------------------------------------------------------------------
+// Operand ring of the register classes: each thread copies its own operands
+// of its next check into shared memory with cp.async while it computes the
+// current one, in two slots that only this thread writes and reads (no
+// barrier; no bank conflicts: a warp's values of one operand are contiguous).
+// The pass is bound by memory once its arithmetic is packed (rate 0.1, n =
+// 10^6, 64 codewords, half: 1.57 GB of DRAM traffic, 0.247 ms for the same
+// loads and stores without arithmetic), and loads held in registers leave
+// too few warps and too much to the order in which the compiler issues them:
+// 0.277-0.299 ms; with the ring 0.257 ms (0.318 ms before both).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t smem_u32(const void *p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+// 16-byte (8-byte) asynchronous copy global -> shared through the load/store
+// unit (both addresses aligned to the size).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// waits until at most N of this thread's committed groups are in flight
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// The update of one check from its terms (read through t), codewords lane0
-// .. lane0+3 of the slab; valid false: compute but store nothing.  sb: the
+constexpr int kRingSlots = 2;
+
+template <typename MsgT, int DC, int DD>
+struct RingShape {
+    using Raw = typename Msg<MsgT>::Raw;
+    static constexpr int kTerms16 = DC + DD;  // posteriors and degree-1 terms, 16 bytes each
+    static constexpr int kStage = kBlock * (kTerms16 * 16 + DC * static_cast<int>(sizeof(Raw)));
+    static constexpr int kBytes = kRingSlots * kStage;
+};
+
+// One thread's operands of one check in a ring slot.
+template <typename MsgT, int DC, int DD>
+struct TermsRing {
+    using S = RingShape<MsgT, DC, DD>;
+    const unsigned char *slot;
+    __device__ __forceinline__ float4 at16(int i) const {
+        return *reinterpret_cast<const float4 *>(slot + (i * kBlock + threadIdx.x) * 16);
+    }
+    __device__ __forceinline__ float4 lv(int i) const { return at16(i); }
+    __device__ __forceinline__ float4 p1(int i) const { return at16(DC + i); }
+    __device__ __forceinline__ typename S::Raw ro(int i) const {
+        return *reinterpret_cast<const typename S::Raw *>(
+            slot + S::kTerms16 * kBlock * 16 + (i * kBlock + threadIdx.x) * sizeof(typename S::Raw));
+    }
+    // requests the operands of a check: its column indices v, the slab's
+    // posteriors, its first message row and degree-1 row
+    template <int W, int N>
+    static __device__ __forceinline__ void request(uint32_t slot, const int32_t (&v)[N], const float *lvb,
+                                                 const MsgT *rp, const float *pp) {
+#pragma unroll
+        for (int i = 0; i < DC; ++i)
+            cp_async16(slot + (i * kBlock + threadIdx.x) * 16, lvb + static_cast<size_t>(v[i]) * W);
+#pragma unroll
+        for (int i = 0; i < DC; ++i) {
+            constexpr uint32_t kRaw = sizeof(typename S::Raw);
+            const uint32_t dst = slot + S::kTerms16 * kBlock * 16 + (i * kBlock + threadIdx.x) * kRaw;
+            if constexpr (kRaw == 16) cp_async16(dst, rp + i * W);
+            else cp_async8(dst, rp + i * W);
+        }
+#pragma unroll
+        for (int i = 0; i < DD; ++i) cp_async16(slot + ((DC + i) * kBlock + threadIdx.x) * 16, pp + i * W);
+    }
+};
+
+// The update of one check, codewords lane0
+// .. lane0+3 of the slab; rout: its first message row there, e0 and s0 its
+// first core edge and degree-1 slot; valid false: compute but store nothing.  sb: the
 // check's syndrome bits for the 4 codewords (bit k: lane0 + k); donenib:
-// their converged flags under early termination.
-template <typename MsgT, int W, int DC, int DD, bool HARD1, bool ACC, bool FUSE, typename Terms>
-__device__ __forceinline__ uint32_t check_terms(const CnArgs &a, int lane0, int slab, bool valid, int32_t e0,
-                                                int32_t s0, uint32_t sb, uint32_t donenib, const Terms &t) {
+// their converged flags under early termination.  FUSE (with kPassHard): with
+// a.fuse the call also returns the previous iteration's syndrome failures of
+// the check for the 4 codewords (bit k: codeword lane0 + k), else 0.  The
+// terms are read through t: lv(i) and ro(i), posterior and stored message of
+// core term i, p1(i), phi term of degree-1 term i.  LAY (layered schedule):
+// the check also owns its core VNs' posteriors and updates them in place.
+template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC, bool FUSE, bool LAY, typename Terms>
+__device__ __forceinline__ uint32_t check_terms(const CnArgs &a, int lane0, int slab, bool valid, MsgT *rout,
+                                                int32_t e0, int32_t s0, uint32_t sb, uint32_t donenib, const Terms &t) {
     constexpr int NB = W / 8;
     constexpr int D = DC + DD;
     constexpr int dc = DC;
+    constexpr bool HARD1 = PASS == kPassHard;
+    const bool deg1_out = HARD1 || (PASS == kPassFull && a.final_pass);
     constexpr int F = DecodeFit<MsgT>::value;
     const float lmax = a.lmax, amin = a.amin;
-    MsgT *rb = static_cast<MsgT *>(a.r) + static_cast<size_t>(slab) * a.e_core * W + lane0;
 
-    // pass 1: f = phi(|q|) carrying the sign of q in its sign bit; the top
-    // bit of par accumulates the sign parity (syndrome bit included).  For a
-    // degree-1 VN q is its channel LLR, whose f was formed once on entry.
-    float f[D][kK];
-    uint32_t par[kK];
-    uint32_t lvs[kK] = {0u, 0u, 0u, 0u};  // sign parity of the posteriors read (fused syndrome)
+    // pass 1: f = phi(|q|) and the signs of q, two codewords at a time; par
+    // accumulates the sign parity (syndrome bits included).  For a degree-1 VN
+    // q is its channel LLR, whose f was formed once on entry.
+    float2 f[D][kP];
+    uint32_t sg[D][kP], par[kP];
+    uint32_t lvs[kP] = {0u, 0u};  // sign parity of the posteriors read (fused syndrome)
 #pragma unroll
-    for (int kk = 0; kk < kK; ++kk) par[kk] = ((sb >> kk) & 1u) << 31;
+    for (int p = 0; p < kP; ++p) par[p] = sign_word_of_bits(sb >> (2 * p));
 #pragma unroll
     for (int i = 0; i < D; ++i) {
         if (i < dc) {
             const float4 lv = t.lv(i);
+            const float2 lp[kP] = {make_float2(lv.x, lv.y), make_float2(lv.z, lv.w)};
             if constexpr (HARD1 && FUSE) {
 #pragma unroll
-                for (int kk = 0; kk < kK; ++kk) lvs[kk] ^= fbits(f4get(lv, kk));
+                for (int p = 0; p < kP; ++p) lvs[p] ^= sign_word(lp[p]);
             }
-            const float4 ro = t.ro(i);
-            const float4 q = make_float4(lv.x - ro.x, lv.y - ro.y, lv.z - ro.z, lv.w - ro.w);
+            const typename Msg<MsgT>::Raw ro = t.ro(i);
             // phi(|q|) floored at amin = phi(lmax) is phi of |q| clamped above at
             // lmax.  |q| is not clamped below: an argument under phi(lmax)
             // gives a term above lmax (up to +inf at 0), which floors every
             // other term's output at amin exactly as the clamped term would;
             // terms are only added, so no inf - inf arises
-            const float4 m = make_float4(fabsf(q.x), fabsf(q.y), fabsf(q.z), fabsf(q.w));
-            const float4 ph = phi4_floor<F>(m, amin);
 #pragma unroll
-            for (int kk = 0; kk < kK; ++kk) {
-                const uint32_t qb = fbits(f4get(q, kk));
-                f[i][kk] = bitsf(fbits(f4get(ph, kk)) | (qb & kSign));
-                par[kk] ^= qb;
+            for (int p = 0; p < kP; ++p) {
+                const float2 q = sub2(lp[p], Msg<MsgT>::pair(ro, p));
+                f[i][p] = phi2_floor<F>(q, amin);
+                sg[i][p] = sign_word(q);
             }
         } else {
-            const float4 p = t.p1(i - dc);
-#pragma unroll
-            for (int kk = 0; kk < kK; ++kk) {
-                f[i][kk] = f4get(p, kk);
-                par[kk] ^= fbits(f[i][kk]);
-            }
+            const float4 v = t.p1(i - dc);
+            f[i][0] = make_float2(fabsf(v.x), fabsf(v.y));
+            f[i][1] = make_float2(fabsf(v.z), fabsf(v.w));
+            sg[i][0] = sign_word(make_float2(v.x, v.y));
+            sg[i][1] = sign_word(make_float2(v.z, v.w));
         }
+#pragma unroll
+        for (int p = 0; p < kP; ++p) par[p] ^= sg[i][p];
     }
-    // exclusive prefix sums of |f| (pre[0], which would be 0, is not formed:
+    // exclusive prefix sums of f (pre[0], which would be 0, is not formed:
     // no addition below has a zero operand)
-    float pre[D][kK];
+    float2 pre[D][kP];
 #pragma unroll
-    for (int kk = 0; kk < kK; ++kk) {
-        if (D >= 2) pre[1][kk] = fabsf(f[0][kk]);
+    for (int p = 0; p < kP; ++p) {
+        if (D >= 2) pre[1][p] = f[0][p];
 #pragma unroll
-        for (int i = 2; i < D; ++i) pre[i][kk] = pre[i - 1][kk] + fabsf(f[i - 1][kk]);
+        for (int i = 2; i < D; ++i) pre[i][p] = add2(pre[i - 1][p], f[i - 1][p]);
     }
     // pass 2 (backwards): leave-one-out sum = prefix + suffix
-    float suf[kK];
+    float2 suf[kP];
 #pragma unroll
     for (int i = D - 1; i >= 0; --i) {
-        if (i < dc || a.final_pass) {
+        if (i < dc || deg1_out) {
             // the output floored at amin is phi of the sum clamped above at
             // lmax.  Every other term is >= amin, so for D >= 3 the sum is at
             // least 2 amin and phi of it stays below lmax; for D <= 2 the
             // output is also clamped above
-            float4 o;
+            float2 o[kP];
 #pragma unroll
-            for (int kk = 0; kk < kK; ++kk) {
-                float v;
-                if (D == 1) v = amin;                      // no other term
-                else if (i == D - 1) v = pre[i][kk];       // no suffix
-                else if (i == 0) v = suf[kk];              // no prefix
-                else v = pre[i][kk] + suf[kk];
-                f4set(o, kk, v);
+            for (int p = 0; p < kP; ++p) {
+                if (D == 1) o[p] = make_float2(amin, amin);     // no other term
+                else if (i == D - 1) o[p] = pre[i][p];          // no suffix
+                else if (i == 0) o[p] = suf[p];                 // no prefix
+                else o[p] = add2(pre[i][p], suf[p]);
             }
             if (HARD1 && i >= dc) {
                 // degree-1 VN, decisions only: the posterior L_ch + r is
@@ -477,46 +576,70 @@ __device__ __forceinline__ uint32_t check_terms(const CnArgs &a, int lane0, int 
                 uint32_t nib = 0;
 #pragma unroll
                 for (int kk = 0; kk < kK; ++kk) {
-                    const uint32_t fb = fbits(f[i][kk]);
-                    const bool l_neg = (fb & kSign) != 0;
-                    const bool r_neg = ((par[kk] ^ fb) & kSign) != 0;
-                    const float fl = fabsf(f[i][kk]), ov = f4get(o, kk);
+                    const bool l_neg = sign_of(sg[i][kk / 2], kk & 1) != 0;
+                    const bool r_neg = sign_of(par[kk / 2] ^ sg[i][kk / 2], kk & 1) != 0;
+                    const float fl = (kk & 1) ? f[i][kk / 2].y : f[i][kk / 2].x;
+                    const float ov = (kk & 1) ? o[kk / 2].y : o[kk / 2].x;
                     const bool neg = (l_neg == r_neg) ? l_neg : (l_neg ? fl < ov : fl > ov);
                     nib |= static_cast<uint32_t>(neg) << kk;
                 }
                 emit_deg1_bits<W>(a, slab, s0 + i - dc, lane0, nib, donenib, valid);
             } else {
-                float4 m = phi4_floor<F>(o, amin);
-                if (D <= 2) m = make_float4(fminf(m.x, lmax), fminf(m.y, lmax), fminf(m.z, lmax), fminf(m.w, lmax));
-                float4 rv;
+                float2 m[kP];
 #pragma unroll
-                for (int kk = 0; kk < kK; ++kk)
-                    f4set(rv, kk, bitsf(fbits(f4get(m, kk)) | ((par[kk] ^ fbits(f[i][kk])) & kSign)));
+                for (int p = 0; p < kP; ++p) {
+                    m[p] = phi2_floor<F>(o[p], amin);
+                    if (D <= 2) m[p] = make_float2(fminf(m[p].x, lmax), fminf(m[p].y, lmax));
+                }
+                const uint32_t w0 = par[0] ^ sg[i][0], w1 = par[1] ^ sg[i][1];
                 if (i < dc) {
                     if (valid) {
-                        MsgT *rp = rb + static_cast<size_t>(e0 + i) * W;
+                        MsgT *rp = rout + i * W;
                         if constexpr (ACC) {
                             // the message as stored joins its VN's posterior
-                            const float4 st = Msg<MsgT>::store_get(rp, rv);
+                            const float4 st = Msg<MsgT>::store_get(rp, with_signs(m[0], m[1], w0, w1));
                             // (the column index is loaded again, an L1 hit, rather than kept
                             // live through both passes)
                             const int32_t v = __ldg(a.col + e0 + i);
                             float *ap = a.acc + (static_cast<size_t>(slab) * a.n_core + v) * W + lane0;
                             atomicAdd(reinterpret_cast<float4 *>(ap), st);
-                        } else if (a.et) {
-                            store_r<MsgT, W, !HARD1>(a, rp, rv, donenib);
+                        } else if constexpr (LAY) {
+                            const typename Msg<MsgT>::Raw raw = t.ro(i);
+                            const float2 r0 = Msg<MsgT>::pair(raw, 0), r1 = Msg<MsgT>::pair(raw, 1);
+                            const float4 lv = t.lv(i);
+                            float4 rv = with_signs(m[0], m[1], w0, w1);
+                            if (donenib) {  // converged lanes keep their messages
+                                if (donenib & 1) rv.x = r0.x;
+                                if (donenib & 2) rv.y = r0.y;
+                                if (donenib & 4) rv.z = r1.x;
+                                if (donenib & 8) rv.w = r1.y;
+                            }
+                            const float4 st = Msg<MsgT>::store_get(rp, rv);
+                            float4 ln = make_float4((lv.x - r0.x) + st.x, (lv.y - r0.y) + st.y, (lv.z - r1.x) + st.z,
+                                                    (lv.w - r1.y) + st.w);
+                            if (donenib) {  // and their posteriors
+                                if (donenib & 1) ln.x = lv.x;
+                                if (donenib & 2) ln.y = lv.y;
+                                if (donenib & 4) ln.z = lv.z;
+                                if (donenib & 8) ln.w = lv.w;
+                            }
+                            const int32_t v = __ldg(a.col + e0 + i);  // (an L1 hit)
+                            float *lp = const_cast<float *>(a.Lv) + (static_cast<size_t>(slab) * a.n_core + v) * W + lane0;
+                            *reinterpret_cast<float4 *>(lp) = ln;
+                        } else if (PASS == kPassFull && donenib) {
+                            store_r<MsgT, W>(a, rp, with_signs(m[0], m[1], w0, w1), donenib);
                         } else {
-                            Msg<MsgT>::store(rp, rv);
+                            Msg<MsgT>::store_signed(rp, m[0], m[1], w0, w1);
                         }
                     }
                 } else {
-                    emit_deg1<MsgT, W>(a, slab, s0 + i - dc, lane0, rv, donenib, valid);
+                    emit_deg1<MsgT, W>(a, slab, s0 + i - dc, lane0, with_signs(m[0], m[1], w0, w1), donenib, valid);
                 }
             }
         }
         if (i > 0) {
 #pragma unroll
-            for (int kk = 0; kk < kK; ++kk) suf[kk] = (i == D - 1) ? fabsf(f[i][kk]) : suf[kk] + fabsf(f[i][kk]);
+            for (int p = 0; p < kP; ++p) suf[p] = (i == D - 1) ? f[i][p] : add2(suf[p], f[i][p]);
         }
     }
     uint32_t fail = 0;
@@ -526,7 +649,7 @@ __device__ __forceinline__ uint32_t check_terms(const CnArgs &a, int lane0, int 
             // (core: posterior < 0, the sign read above; degree-1: stored bit)
             uint32_t x = sb & 0xFu;
 #pragma unroll
-            for (int kk = 0; kk < kK; ++kk) x ^= (lvs[kk] >> 31) << kk;
+            for (int kk = 0; kk < kK; ++kk) x ^= (sign_of(lvs[kk / 2], kk & 1) >> 31) << kk;
             if (DD == 1)
                 x ^= (static_cast<uint32_t>(a.hb1_prev[(static_cast<size_t>(slab) * a.n_deg1 + s0) * NB + lane0 / 8]) >>
                       (lane0 & 7)) & 0xFu;
@@ -621,47 +744,103 @@ __device__ __forceinline__ void check_irregular(const CnArgs &a, const ClassLaun
     }
 }
 
-// Classes of at most 6 terms loop over their checks on a capped grid: a
-// thread's set-up (indices, slab bases) is then shared by several checks.
-// The 7- and 8-term classes (80 registers) take one check per thread.
-template <int D> constexpr bool kLoopedClass = D <= 6;
+// Blocks per SM of a register class's check kernel (128 registers for six
+// terms, so that nothing spills) and waves of its grid.  Measured (check pass,
+// n = 10^6, 64 codewords, half): six terms at 3 / 4 / 5 blocks 0.296 / 0.285 /
+// 0.296 ms, four terms at 4 / 5 / 6 blocks 0.199 / 0.197 / 0.193 ms, three at
+// 6 / 7 / 8 blocks 0.148 / 0.154 / 0.149 ms; four waves instead of two +1 %.
+template <int D>
+constexpr int kCheckBlocksPerSm = D > 6 ? 3 : D > 4 ? 4 : D == 4 ? 6 : 8;
+constexpr int kCheckWaves = 2;
+inline int check_blocks_per_sm(int deg) {
+    return deg > 6 ? kCheckBlocksPerSm<7> : deg > 4 ? kCheckBlocksPerSm<6> : deg == 4 ? kCheckBlocksPerSm<4>
+                                                                                     : kCheckBlocksPerSm<3>;
+}
+// Grid width of a class launch: the threads step through the class's checks.
+inline int class_blocks(const ClassLaunch &cl, int sm_count) {
+    return std::max(1, std::min(cl.blocks, sm_count * kCheckWaves * check_blocks_per_sm(cl.deg)));
+}
+// Above the default limit of dynamic shared memory a kernel has to opt in
+// (float messages, 7 and 8 terms).
+template <int BYTES, typename K>
+void allow_smem(K kernel) {
+    if constexpr (BYTES > 48 * 1024)
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BYTES);
+}
 
 // The threads of a class launch (t0: thread index in the slab's grid of
-// `blocks` blocks): looped classes step through their checks, the others take
-// one; with HARD1 the fused syndrome failures are ORed into a.fail_prev.
-template <typename MsgT, int W, int DC, int DD, bool HARD1, bool ACC = false, bool FUSE = HARD1>
+// `blocks` blocks; smem: RingShape::kBytes bytes), each taking every
+// stride-th check with the same codewords; both threads of a shuffle pair
+// belong to one check and leave together.  With FUSE the fused syndrome
+// failures are ORed into a.fail_prev.  LAY: the launch's k-th check is
+// pos[k], its messages start at layered edge cl.e0 + k DC (contiguous in the
+// launch), its degree-1 slots follow the class order.
+template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC = false, bool FUSE = false, bool LAY = false>
 __device__ __forceinline__ void check_class_body(const CnArgs &a, const ClassLaunch &cl, int64_t t0,
-                                                 int32_t blocks, int slab) {
+                                                 int32_t blocks, int slab, unsigned char *smem,
+                                                 const int32_t *pos = nullptr) {
+    using Ring = TermsRing<MsgT, DC, DD>;
+    constexpr int kStage = RingShape<MsgT, DC, DD>::kStage;
     constexpr int TPC = W / kK;
+    constexpr int NB = W / 8;
     const int lane0 = static_cast<int>(t0 % TPC) * kK;
+    MsgT *rb = static_cast<MsgT *>(a.r) + (static_cast<size_t>(slab) * a.e_core + cl.e0) * W + lane0;
+    const float *lvb = a.Lv + static_cast<size_t>(slab) * a.n_core * W + lane0;
+    const float *pb = a.phi1 + (static_cast<size_t>(slab) * a.n_deg1 + cl.s0) * W + lane0;
+    const uint8_t *sbp = a.sbits + (static_cast<size_t>(slab) * a.n_cn + cl.c0) * NB + lane0 / 8;
+    const uint32_t donenib = (PASS != kPassPlain && a.et) ? done_nibble<W>(a.done, slab, lane0) : 0u;
+    const int32_t stride = blocks * (kBlock / TPC);
+    const uint32_t sm = smem_u32(smem);
+    int32_t v[DC > 0 ? DC : 1];  // column indices of the check whose operands are requested next,
+    int32_t cn = 0;              // and its position in the class
+    uint32_t sbn = 0;            // syndrome byte of the check requested last
+    auto cols = [&](int32_t j) {
+        j = min(j, cl.count - 1);  // (past the end: a valid address that nothing uses)
+#pragma unroll
+        for (int i = 0; i < DC; ++i) v[i] = __ldg(a.col + cl.e0 + j * DC + i);
+        cn = LAY ? __ldg(pos + j) - cl.c0 : j;
+    };
+    auto request = [&](int32_t j, int slot) {
+        if (j < cl.count) {
+            Ring::template request<W>(sm + slot * kStage, v, lvb, rb + static_cast<size_t>(j * DC) * W,
+                                      pb + static_cast<size_t>(cn * DD) * W);
+            sbn = sbp[static_cast<size_t>(cn) * NB];
+        }
+        cp_async_commit();  // (an empty group past the end keeps the count)
+    };
     uint32_t fail = 0;
-    if constexpr (kLoopedClass<DC + DD>) {
-        // a capped grid; each thread takes every stride-th check with the
-        // same lanes, so its set-up is shared by several checks.  Both
-        // threads of a shuffle pair belong to one check and leave together.
-        const int32_t jstride = blocks * (kBlock / TPC);
-        for (int32_t j = static_cast<int32_t>(t0 / TPC); j < cl.count; j += jstride)
-            fail |= check_regular<MsgT, W, DC, DD, HARD1, ACC, FUSE>(a, cl, j, lane0, slab);
-    } else {
-        fail = check_regular<MsgT, W, DC, DD, HARD1, ACC, FUSE>(a, cl, static_cast<int32_t>(t0 / TPC), lane0, slab);
+    int32_t j = static_cast<int32_t>(t0 / TPC);
+    cols(j);
+    request(j, 0);
+    int32_t c = cn;
+    cols(j + stride);
+    for (int slot = 0; j < cl.count; j += stride, slot ^= 1) {
+        const uint32_t sb = sbn >> (lane0 & 7);
+        const int32_t s0 = cl.s0 + c * DD;
+        request(j + stride, slot ^ 1);
+        c = cn;
+        cols(j + 2 * stride);
+        cp_async_wait<1>();
+        const Ring t{smem + slot * kStage};
+        fail |= check_terms<MsgT, W, DC, DD, PASS, ACC, FUSE, LAY>(
+            a, lane0, slab, true, rb + static_cast<size_t>(j * DC) * W, cl.e0 + j * DC, s0, sb, donenib, t);
     }
-    if constexpr (HARD1 && FUSE) {
+    if constexpr (FUSE) {
         if (a.fuse) flush_fail<W>(a.fail_prev + slab * ((W + 31) / 32), fail, lane0);
     }
 }
 
 // One check class per launch, its shape (DC, DD) a compile-time constant: the
 // register arrays are sized exactly and only this class's code is hot.
-// HARD1 without FUSE (decisions only, the syndrome checked by its own
-// kernel): 7 blocks per SM, 72 registers without spills.
-template <typename MsgT, int W, int DC, int DD, bool HARD1, bool ACC = false, bool FUSE = HARD1>
-__global__ void __launch_bounds__(kBlock, (DC + DD <= 6 ? ((ACC || (HARD1 && !FUSE)) ? 7 : 8) : 6))
+template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC = false, bool FUSE = false>
+__global__ void __launch_bounds__(kBlock, (kCheckBlocksPerSm<DC + DD>))
     k_check_update(CnArgs a, ClassLaunch cl) {
     const int slab = blockIdx.y;
-    if (a.et && slab_all_done<W>(a.done, slab)) return;  // block-uniform
-    check_class_body<MsgT, W, DC, DD, HARD1, ACC, FUSE>(a, cl,
+    if (PASS != kPassPlain && a.et && slab_all_done<W>(a.done, slab)) return;  // block-uniform
+    extern __shared__ __align__(128) unsigned char smem[];
+    check_class_body<MsgT, W, DC, DD, PASS, ACC, FUSE>(a, cl,
                                                   static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x,
-                                                  static_cast<int32_t>(gridDim.x), slab);
+                                                  static_cast<int32_t>(gridDim.x), slab, smem);
 }
 
 // ---------------------------------------------------------------------------
@@ -680,9 +859,6 @@ __global__ void __launch_bounds__(kBlock, (DC + DD <= 6 ? ((ACC || (HARD1 && !FU
 constexpr int kStagedBlocksPerSm = 6;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
@@ -736,11 +912,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         : "memory");
 }
 
-// 16-byte asynchronous copy global -> shared through the load/store unit
-// (both addresses 16-byte aligned).
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
 // Arrive on the mbarrier once this thread's earlier cp.async copies have
 // landed; counts as one of the phase's expected arrivals.
 __device__ __forceinline__ void cp_async_arrive_noinc(uint64_t *bar) {
@@ -769,7 +940,9 @@ struct TermsShared {
     const MsgT *msg;
     const float *phi;
     __device__ __forceinline__ float4 lv(int i) const { return *reinterpret_cast<const float4 *>(post + i * W); }
-    __device__ __forceinline__ float4 ro(int i) const { return Msg<MsgT>::load(msg + i * W); }
+    __device__ __forceinline__ typename Msg<MsgT>::Raw ro(int i) const {
+        return *reinterpret_cast<const typename Msg<MsgT>::Raw *>(msg + i * W);
+    }
     __device__ __forceinline__ float4 p1(int i) const { return *reinterpret_cast<const float4 *>(phi + i * W); }
 };
 
@@ -854,7 +1027,7 @@ __global__ void __launch_bounds__(kBlock, kStagedBlocksPerSm) k_check_staged(CnA
             float *post = reinterpret_cast<float *>(base + S::kMsg + S::kP1) + g * DC * W + lane0;
 #pragma unroll
             for (int i = 0; i < DC; ++i)
-                if (v[i] >= 0) cp_async16(post + i * W, lvsrc + static_cast<size_t>(v[i]) * W + lane0);
+                if (v[i] >= 0) cp_async16(smem_u32(post + i * W), lvsrc + static_cast<size_t>(v[i]) * W + lane0);
             cp_async_arrive_noinc(&full[buf]);
         } else {
             if (v[0] >= 0) {
@@ -890,8 +1063,9 @@ __global__ void __launch_bounds__(kBlock, kStagedBlocksPerSm) k_check_staged(CnA
         t.msg = reinterpret_cast<const MsgT *>(base) + g * DC * W + lane0;
         t.phi = reinterpret_cast<const float *>(base + S::kMsg) + g * DD * W + lane0;
         t.post = reinterpret_cast<const float *>(base + S::kMsg + S::kP1) + g * DC * W + lane0;
-        check_terms<MsgT, W, DC, DD, false, false, false>(a, lane0, slab, valid, cl.e0 + j * DC, cl.s0 + j * DD, sb,
-                                                   donenib, t);
+        MsgT *rout = static_cast<MsgT *>(a.r) + (static_cast<size_t>(slab) * a.e_core + cl.e0 + j * DC) * W + lane0;
+        check_terms<MsgT, W, DC, DD, kPassFull, false, false, false>(a, lane0, slab, valid, rout, cl.e0 + j * DC,
+                                                              cl.s0 + j * DD, sb, donenib, t);
         if (__syncthreads_or(!ok)) {
             // a copy never completed: record it, give the copies in flight
             // (this stage's and the next one's) a bounded time to land, leave
@@ -924,9 +1098,8 @@ __global__ void __launch_bounds__(kBlock) k_check_update_irregular(CnArgs a, Cla
 // Classes with at most one degree-1 VN per check and at most kMaxRegDeg terms
 // run the register kernel for their shape; any other class (possible in
 // caller graphs, not in the MET ensembles) runs the streaming kernel.
-// cap_blocks: grid width for the looped classes (a few waves of the GPU);
 // hard1: early termination without soft output (degree-1 decisions only, and
-// the fused syndrome check when ca.fuse; see check_regular).  With ca.acc set
+// the fused syndrome check when ca.fuse; see check_terms).  With ca.acc set
 // (fixed iterations, default slab width, register classes only) the kernels
 // also add every new message to the next posteriors.
 template <typename MsgT, int W>
@@ -994,33 +1167,36 @@ bool try_launch_staged(const CnArgs &ca, const ClassLaunch &cl, int slabs, cudaS
 }
 
 template <typename MsgT, int W>
-void launch_check_class(const CnArgs &ca, const ClassLaunch &cl, int slabs, cudaStream_t st, int cap_blocks,
+void launch_check_class(const CnArgs &ca, const ClassLaunch &cl, int slabs, cudaStream_t st, int sm_count,
                         bool hard1, int staged_cap = 0, int staged_mode = MLD_STAGE_DIRECT) {
     if (ca.rule == kRuleMinSum) {
-        launch_minsum_class<MsgT, W>(ca, cl, slabs, st, cap_blocks);
+        launch_minsum_class<MsgT, W>(ca, cl, slabs, st, sm_count * 16);
         return;
     }
     if (try_launch_staged<MsgT, W>(ca, cl, slabs, st, staged_cap, hard1, staged_mode)) return;
     const dim3 grid(cl.blocks, slabs);
-    const dim3 capped(std::max(1, std::min(cl.blocks, cap_blocks)), slabs);
-    const dim3 g = (cl.dc >= 0 && cl.deg <= 6) ? capped : grid;
-    // the decisions-only kernels without the fused syndrome run 7 blocks per
-    // SM: their looped grid is two waves of 7
-    const dim3 capped7(std::max(1, std::min(cl.blocks, cap_blocks / 8 * 7)), slabs);
-    const dim3 g7 = (cl.dc >= 0 && cl.deg <= 6) ? capped7 : grid;
     const int dd = cl.deg - cl.dc;
+    const bool plain = !ca.et && !ca.final_pass;
+#define MLD_LAUNCH(DCV, DDV, ...)                                                                   \
+    do {                                                                                            \
+        constexpr int bytes = RingShape<MsgT, DCV, DDV>::kBytes;                                    \
+        allow_smem<bytes>(k_check_update<MsgT, W, DCV, DDV, __VA_ARGS__>);                          \
+        k_check_update<MsgT, W, DCV, DDV, __VA_ARGS__>                                              \
+            <<<dim3(class_blocks(cl, sm_count), slabs), kBlock, bytes, st>>>(ca, cl);               \
+    } while (0)
 #define MLD_CASE(DCV, DDV)                                                                          \
     case (DCV) * 2 + (DDV):                                                                         \
-        static_assert(kLoopedClass<(DCV) + (DDV)> == ((DCV) + (DDV) <= 6), "grid choice");         \
         if constexpr (kAccWidth<MsgT, W>) {                                                         \
             if (ca.acc) {                                                                           \
-                k_check_update<MsgT, W, DCV, DDV, false, true><<<g, kBlock, 0, st>>>(ca, cl);      \
+                if (plain) MLD_LAUNCH(DCV, DDV, kPassPlain, true);                                  \
+                else MLD_LAUNCH(DCV, DDV, kPassFull, true);                                         \
                 return;                                                                             \
             }                                                                                       \
         }                                                                                           \
-        if (hard1 && ca.fuse) k_check_update<MsgT, W, DCV, DDV, true><<<g, kBlock, 0, st>>>(ca, cl); \
-        else if (hard1) k_check_update<MsgT, W, DCV, DDV, true, false, false><<<g7, kBlock, 0, st>>>(ca, cl); \
-        else k_check_update<MsgT, W, DCV, DDV, false><<<g, kBlock, 0, st>>>(ca, cl);              \
+        if (hard1 && ca.fuse) MLD_LAUNCH(DCV, DDV, kPassHard, false, true);                         \
+        else if (hard1) MLD_LAUNCH(DCV, DDV, kPassHard);                                            \
+        else if (plain) MLD_LAUNCH(DCV, DDV, kPassPlain);                                           \
+        else MLD_LAUNCH(DCV, DDV, kPassFull);                                                       \
         return;
     if (cl.dc >= 0 && (dd == 0 || dd == 1)) {
         switch (cl.dc * 2 + dd) {
@@ -1032,6 +1208,7 @@ void launch_check_class(const CnArgs &ca, const ClassLaunch &cl, int slabs, cuda
         }
     }
 #undef MLD_CASE
+#undef MLD_LAUNCH
     k_check_update_irregular<MsgT, W><<<grid, kBlock, 0, st>>>(ca, cl);
 }
 
@@ -1048,11 +1225,11 @@ __device__ __forceinline__ void pdl_enter() {
 }
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args) {
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1067,154 +1244,21 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStre
 // from the latest messages.  The checks of a layer share no core VN, so a
 // check owns the posteriors of its core VNs while its layer runs: it forms
 // q = L_v - r_old (Eq. 4 with the current messages), the new r (Eqs. 2-3,
-// as in check_regular) and L_v <- (L_v - r_old) + r_new in place.
+// check_terms) and L_v <- (L_v - r_old) + r_new in place.  A launch's checks
+// go through the operand ring: no other check of the launch writes the rows
+// that a thread has requested ahead (posteriors are copied past L1, which is
+// not coherent between SMs).
 // ---------------------------------------------------------------------------
-// Layered launches number their messages contiguously: the launch's k-th
-// check (internal id c) owns layered edges cl.e0 + k DC ..; a.col is the
-// layered column table.  Its degree-1 slots follow the class order.  HARD1:
-// a degree-1 VN gets its decision only (early termination without soft
-// output), as in check_terms.
-template <typename MsgT, int W, int DC, int DD, bool HARD1 = false>
-__device__ __forceinline__ void check_layered(const CnArgs &a, const ClassLaunch &cl, int32_t c, int32_t k,
-                                              int lane0, int slab, bool valid) {
-    constexpr int D = DC + DD;
-    constexpr int F = DecodeFit<MsgT>::value;
-    constexpr int NB = W / 8;
-    const int32_t e0 = cl.e0 + k * DC;
-    const int32_t s0 = cl.s0 + (c - cl.c0) * DD;
-    const float lmax = a.lmax, amin = a.amin;
-    const uint32_t sb =
-        (static_cast<uint32_t>(a.sbits[(static_cast<size_t>(slab) * a.n_cn + c) * NB + lane0 / 8]) >>
-         (lane0 & 7));
-    const uint32_t donenib = a.et ? done_nibble<W>(a.done, slab, lane0) : 0u;
-    MsgT *rb = static_cast<MsgT *>(a.r) + static_cast<size_t>(slab) * a.e_core * W + lane0;
-    // the posteriors are written by this kernel: plain (coherent) loads
-    float *lvb = const_cast<float *>(a.Lv) + static_cast<size_t>(slab) * a.n_core * W + lane0;
-    const float *p1b = a.phi1 + static_cast<size_t>(slab) * a.n_deg1 * W + lane0;
-
-    float f[D][kK];
-    uint32_t par[kK];
-#pragma unroll
-    for (int kk = 0; kk < kK; ++kk) par[kk] = ((sb >> kk) & 1u) << 31;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-        if (i < DC) {
-            const int32_t v = __ldg(a.col + e0 + i);
-            const float4 lv = *reinterpret_cast<const float4 *>(lvb + static_cast<size_t>(v) * W);
-            const float4 ro = Msg<MsgT>::load(rb + static_cast<size_t>(e0 + i) * W);
-            const float4 q = make_float4(lv.x - ro.x, lv.y - ro.y, lv.z - ro.z, lv.w - ro.w);
-            const float4 m = make_float4(fabsf(q.x), fabsf(q.y), fabsf(q.z), fabsf(q.w));
-            const float4 ph = phi4_floor<F>(m, amin);
-#pragma unroll
-            for (int kk = 0; kk < kK; ++kk) {
-                const uint32_t qb = fbits(f4get(q, kk));
-                f[i][kk] = bitsf(fbits(f4get(ph, kk)) | (qb & kSign));
-                par[kk] ^= qb;
-            }
-        } else {
-            const float4 p = ldf4(p1b + static_cast<size_t>(s0 + i - DC) * W);
-#pragma unroll
-            for (int kk = 0; kk < kK; ++kk) {
-                f[i][kk] = f4get(p, kk);
-                par[kk] ^= fbits(f[i][kk]);
-            }
-        }
-    }
-    float pre[D][kK];
-#pragma unroll
-    for (int kk = 0; kk < kK; ++kk) {
-        if (D >= 2) pre[1][kk] = fabsf(f[0][kk]);
-#pragma unroll
-        for (int i = 2; i < D; ++i) pre[i][kk] = pre[i - 1][kk] + fabsf(f[i - 1][kk]);
-    }
-    float suf[kK];
-#pragma unroll
-    for (int i = D - 1; i >= 0; --i) {
-        if (i < DC || a.final_pass) {
-            float4 o;
-#pragma unroll
-            for (int kk = 0; kk < kK; ++kk) {
-                float v;
-                if (D == 1) v = amin;
-                else if (i == D - 1) v = pre[i][kk];
-                else if (i == 0) v = suf[kk];
-                else v = pre[i][kk] + suf[kk];
-                f4set(o, kk, v);
-            }
-            if (HARD1 && i >= DC) {
-                // decision of L_ch + r without r: see check_terms
-                uint32_t nib = 0;
-#pragma unroll
-                for (int kk = 0; kk < kK; ++kk) {
-                    const uint32_t fb = fbits(f[i][kk]);
-                    const bool l_neg = (fb & kSign) != 0;
-                    const bool r_neg = ((par[kk] ^ fb) & kSign) != 0;
-                    const float fl = fabsf(f[i][kk]), ov = f4get(o, kk);
-                    const bool neg = (l_neg == r_neg) ? l_neg : (l_neg ? fl < ov : fl > ov);
-                    nib |= static_cast<uint32_t>(neg) << kk;
-                }
-                emit_deg1_bits<W>(a, slab, s0 + i - DC, lane0, nib, donenib, valid);
-            } else {
-            float4 mm = phi4_floor<F>(o, amin);
-            if (D <= 2) mm = make_float4(fminf(mm.x, lmax), fminf(mm.y, lmax), fminf(mm.z, lmax), fminf(mm.w, lmax));
-            float4 rv;
-#pragma unroll
-            for (int kk = 0; kk < kK; ++kk)
-                f4set(rv, kk, bitsf(fbits(f4get(mm, kk)) | ((par[kk] ^ fbits(f[i][kk])) & kSign)));
-            if (i < DC) {
-                if (valid) {
-                    MsgT *rp = rb + static_cast<size_t>(e0 + i) * W;
-                    const float4 ro = Msg<MsgT>::load(rp);
-                    if (donenib) {  // converged lanes keep their messages
-                        if (donenib & 1) rv.x = ro.x;
-                        if (donenib & 2) rv.y = ro.y;
-                        if (donenib & 4) rv.z = ro.z;
-                        if (donenib & 8) rv.w = ro.w;
-                    }
-                    const float4 st = Msg<MsgT>::store_get(rp, rv);
-                    float *lp = lvb + static_cast<size_t>(__ldg(a.col + e0 + i)) * W;
-                    const float4 lv = *reinterpret_cast<const float4 *>(lp);
-                    float4 ln = make_float4((lv.x - ro.x) + st.x, (lv.y - ro.y) + st.y, (lv.z - ro.z) + st.z,
-                                            (lv.w - ro.w) + st.w);
-                    if (donenib) {  // and their posteriors
-                        if (donenib & 1) ln.x = lv.x;
-                        if (donenib & 2) ln.y = lv.y;
-                        if (donenib & 4) ln.z = lv.z;
-                        if (donenib & 8) ln.w = lv.w;
-                    }
-                    *reinterpret_cast<float4 *>(lp) = ln;
-                }
-            } else {
-                emit_deg1<MsgT, W>(a, slab, s0 + i - DC, lane0, rv, donenib, valid);
-            }
-            }
-        }
-        if (i > 0) {
-#pragma unroll
-            for (int kk = 0; kk < kK; ++kk) suf[kk] = (i == D - 1) ? fabsf(f[i][kk]) : suf[kk] + fabsf(f[i][kk]);
-        }
-    }
-}
-
-// One layer's checks of one class (pos[k]: internal id of the k-th), on a
-// capped grid: a thread keeps its lanes and steps through every stride-th
-// check, so consecutive checks of a wave read consecutive message rows.
-// Both threads of a shuffle pair belong to one check and leave together.
-// Blocks per SM of the layered kernels (72 registers per thread).
-constexpr int kLayeredBlocksPerSm = 7;
-
-template <typename MsgT, int W, int DC, int DD, bool HARD1>
-__global__ void __launch_bounds__(kBlock, (DC + DD <= 6 ? kLayeredBlocksPerSm : 6))
+template <typename MsgT, int W, int DC, int DD, int PASS>
+__global__ void __launch_bounds__(kBlock, (kCheckBlocksPerSm<DC + DD>))
     k_check_layered(CnArgs a, ClassLaunch cl, const int32_t *pos) {
-    constexpr int TPC = W / kK;
     pdl_enter();  // the previous layer's messages and posteriors
     const int slab = blockIdx.y;
-    if (a.et && slab_all_done<W>(a.done, slab)) return;  // block-uniform
-    const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int lane0 = static_cast<int>(t % TPC) * kK;
-    const int32_t kstride = static_cast<int32_t>(gridDim.x) * (kBlock / TPC);
-    for (int32_t k = static_cast<int32_t>(t / TPC); k < cl.count; k += kstride)
-        check_layered<MsgT, W, DC, DD, HARD1>(a, cl, __ldg(pos + k), k, lane0, slab, true);
+    if (PASS != kPassPlain && a.et && slab_all_done<W>(a.done, slab)) return;  // block-uniform
+    extern __shared__ __align__(128) unsigned char smem[];
+    check_class_body<MsgT, W, DC, DD, PASS, false, false, true>(
+        a, cl, static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x, static_cast<int32_t>(gridDim.x), slab, smem,
+        pos);
 }
 
 // Layered update of a check of any degree (edges read through cptr/dptr);
@@ -1313,6 +1357,12 @@ __global__ void __launch_bounds__(kBlock) k_check_layered_irregular(CnArgs a, Cl
         check_layered_irregular<MsgT, W>(a, __ldg(pos + k), k, lane0, slab);
 }
 
+// Grid width of a layered launch: one wave.
+inline int layer_blocks(int64_t blocks, int deg, int sm_count) {
+    const int per_sm = deg < 0 ? 7 : check_blocks_per_sm(deg);
+    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(blocks, static_cast<int64_t>(sm_count) * per_sm)));
+}
+
 // The layered schedule is built for the default slab width of each message
 // type.  Classes of at most 8 terms with at most one degree-1 VN run the
 // register kernel of their shape, any other class the runtime-degree kernel.
@@ -1322,10 +1372,18 @@ void launch_layered(const CnArgs &ca, const ClassLaunch &cl, const int32_t *pos,
     if constexpr (kAccWidth<MsgT, W>) {
         const dim3 grid(cl.blocks, slabs);
         const int dd = cl.deg - cl.dc;
-#define MLD_LCASE(DCV, DDV)                                                                          \
-    case (DCV) * 2 + (DDV):                                                                          \
-        if (hard1) launch_pdl(k_check_layered<MsgT, W, DCV, DDV, true>, grid, dim3(kBlock), st, ca, cl, pos); \
-        else launch_pdl(k_check_layered<MsgT, W, DCV, DDV, false>, grid, dim3(kBlock), st, ca, cl, pos);     \
+        const bool plain = !ca.et && !ca.final_pass;
+#define MLD_LLAUNCH(DCV, DDV, PASS)                                                                 \
+    do {                                                                                            \
+        constexpr int bytes = RingShape<MsgT, DCV, DDV>::kBytes;                                    \
+        allow_smem<bytes>(k_check_layered<MsgT, W, DCV, DDV, PASS>);                                \
+        launch_pdl(k_check_layered<MsgT, W, DCV, DDV, PASS>, grid, dim3(kBlock), bytes, st, ca, cl, pos); \
+    } while (0)
+#define MLD_LCASE(DCV, DDV)                                                                         \
+    case (DCV) * 2 + (DDV):                                                                         \
+        if (hard1) MLD_LLAUNCH(DCV, DDV, kPassHard);                                                \
+        else if (plain) MLD_LLAUNCH(DCV, DDV, kPassPlain);                                          \
+        else MLD_LLAUNCH(DCV, DDV, kPassFull);                                                      \
         return;
         if (cl.dc >= 0 && (dd == 0 || dd == 1)) {
             switch (cl.dc * 2 + dd) {
@@ -1337,7 +1395,8 @@ void launch_layered(const CnArgs &ca, const ClassLaunch &cl, const int32_t *pos,
             }
         }
 #undef MLD_LCASE
-        launch_pdl(k_check_layered_irregular<MsgT, W>, grid, dim3(kBlock), st, ca, cl, pos);
+#undef MLD_LLAUNCH
+        launch_pdl(k_check_layered_irregular<MsgT, W>, grid, dim3(kBlock), 0, st, ca, cl, pos);
     }
 }
 

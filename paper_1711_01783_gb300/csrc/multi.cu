@@ -61,19 +61,19 @@ __device__ __forceinline__ CnArgs job_cn(const JobDev &j, const Seg &sg, int32_t
     return a;
 }
 
-// The decisions-only form (with the fused syndrome) runs 7 blocks per SM:
-// at 8 its posterior-sign bookkeeping spills.
-template <typename MsgT, int W, int DC, int DD, bool HARD1>
-__global__ void __launch_bounds__(kBlock, (DC + DD <= 6 ? (HARD1 ? 7 : 8) : 6))
+// The decisions-only form carries the fused syndrome.
+template <typename MsgT, int W, int DC, int DD, int PASS>
+__global__ void __launch_bounds__(kBlock, (kCheckBlocksPerSm<DC + DD>))
     km_check(const JobDev *jobs, const Seg *segs, int nseg, int32_t l) {
     const Seg sg = segs[find_seg(segs, nseg)];
     const CnArgs a = job_cn<W>(jobs[sg.job], sg, l);
     const int local = blockIdx.x - sg.block0;
     const int slab = local / sg.bps;
     if (a.et && slab_all_done<W>(a.done, slab)) return;
-    // the segment's grid is capped for looped classes (build_plan)
-    check_class_body<MsgT, W, DC, DD, HARD1>(a, sg.cl, static_cast<int64_t>(local % sg.bps) * blockDim.x + threadIdx.x,
-                                             sg.bps, slab);
+    // the segment's grid is capped for register classes (build_plan)
+    extern __shared__ __align__(128) unsigned char smem[];
+    check_class_body<MsgT, W, DC, DD, PASS, false, PASS == kPassHard>(
+        a, sg.cl, static_cast<int64_t>(local % sg.bps) * blockDim.x + threadIdx.x, sg.bps, slab, smem);
 }
 
 template <typename MsgT, int W>
@@ -155,7 +155,7 @@ enum OpKind { kOpMemset, kOpInterleave, kOpSynIn, kOpHard, kOpCheck, kOpVar, kOp
 
 struct Op {
     int kind = 0, half = 0, W = 0, dc = 0, dd = 0, parity = 0;
-    int hard1 = 0;  // check ops: degree-1 decisions only
+    int pass = 0;  // check ops: kPass*
     int32_t l = 0;
     int seg0 = 0, nseg = 0, blocks = 0;
     // memset / hard-decision ops
@@ -188,8 +188,16 @@ void launch_check_op(const mld_plan *p, const Op &op, cudaStream_t st) {
     const Seg *S = p->d_segs + op.seg0;
 #define MLD_CASE(DCV, DDV)                                                                          \
     if (op.dc == (DCV) && op.dd == (DDV)) {                                                         \
-        if (op.hard1) km_check<MsgT, W, DCV, DDV, true><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg, op.l); \
-        else km_check<MsgT, W, DCV, DDV, false><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg, op.l);      \
+        constexpr int sm = RingShape<MsgT, DCV, DDV>::kBytes;                                      \
+        if (op.pass == kPassHard) allow_smem<sm>(km_check<MsgT, W, DCV, DDV, kPassHard>);           \
+        else if (op.pass == kPassPlain) allow_smem<sm>(km_check<MsgT, W, DCV, DDV, kPassPlain>);    \
+        else allow_smem<sm>(km_check<MsgT, W, DCV, DDV, kPassFull>);                                \
+        if (op.pass == kPassHard)                                                                   \
+            km_check<MsgT, W, DCV, DDV, kPassHard><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.l); \
+        else if (op.pass == kPassPlain)                                                             \
+            km_check<MsgT, W, DCV, DDV, kPassPlain><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.l); \
+        else                                                                                        \
+            km_check<MsgT, W, DCV, DDV, kPassFull><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.l); \
         return;                                                                                     \
     }
     MLD_CASE(1, 0) MLD_CASE(2, 0) MLD_CASE(3, 0) MLD_CASE(4, 0)
@@ -299,7 +307,7 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
     }
 
     // one op per group key; segments of the group are the jobs' shares
-    using Key = std::tuple<int, int, int, int, int, int>;  // kind, half, W, dc, dd, hard1
+    using Key = std::tuple<int, int, int, int, int, int>;  // kind, half, W, dc, dd, pass
     auto flush = [&](std::map<Key, std::vector<Seg>> &groups, int32_t l, int parity) {
         for (auto &kv : groups) {
             Op op;
@@ -308,7 +316,7 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
             op.W = std::get<2>(kv.first);
             op.dc = std::get<3>(kv.first);
             op.dd = std::get<4>(kv.first);
-            op.hard1 = std::get<5>(kv.first);
+            op.pass = std::get<5>(kv.first);
             op.l = l;
             op.parity = parity;
             op.seg0 = static_cast<int>(segs.size());
@@ -424,14 +432,10 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
             for (const ClassLaunch &cl : d->g->launches[width_index(d->W)]) {
                 const int dd = cl.deg - cl.dc;
                 const bool regular = cl.dc >= 0 && (dd == 0 || dd == 1);
-                // looped register classes (at most 6 terms) run on a capped
-                // grid of two waves (7 blocks per SM for the decisions-only form)
-                const bool looped = regular && cl.deg <= 6;
-                const int hard1 = (hard1_job(j) && regular) ? 1 : 0;
-                const int cap = sm_count * (hard1 ? 14 : 16);
-                Seg s = seg(j, looped ? std::max(1, std::min(cl.blocks, cap)) : cl.blocks, jd[j].slabs, fl);
+                const int pass = !regular ? kPassFull : hard1_job(j) ? kPassHard : (fl & 1) ? kPassFull : kPassPlain;
+                Seg s = seg(j, regular ? class_blocks(cl, sm_count) : cl.blocks, jd[j].slabs, fl);
                 s.cl = cl;
-                groups[Key{kOpCheck, half, d->W, regular ? cl.dc : -1, regular ? dd : -1, hard1}].push_back(s);
+                groups[Key{kOpCheck, half, d->W, regular ? cl.dc : -1, regular ? dd : -1, pass}].push_back(s);
             }
             if (fused_job(j) && l >= 2) lanes.push_back(j);
         }
