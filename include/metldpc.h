@@ -208,7 +208,9 @@ int mld_peg_edges(int32_t n_vn, int32_t n_types, const int32_t *deg, int32_t n_c
  *   lmax       : LLR clamp (> 0; 0 selects 25).  Channel LLRs, messages and
  *                the arguments of phi are kept within it (see mld_decode).
  *   slab_width : 8, 16, 32 or 64 codewords per slab; 0 selects 32 for F32
- *                and 64 for F16.
+ *                and 64 for F16, and lets a flooding sum-product gather decode
+ *                of fewer codewords run in the narrowest slab that holds them
+ *                (same results).
  *   vn_update  : how the variable update of Eq. 4 forms the posteriors
  *                L_v = L_ch(v) + sum_{e in C_v} r_e:
  *                MLD_VN_GATHER (0, default): a separate pass gathers each
@@ -368,7 +370,8 @@ int mld_decoder_test_stall(mld_decoder *d, int32_t bytes);
  * Semantics per codeword are those of mld_decode_y / mld_decode with the
  * job's max_iters; with MLD_EARLY_TERM each codeword stops at its first
  * syndrome match (Methods, Step 5) and a slab whose codewords have all
- * stopped is skipped.
+ * stopped is skipped; the iterations are then a loop inside the graph, which
+ * the device leaves once every codeword has stopped.
  *   decoder    : from mld_decoder_create; at most one job per decoder.
  *   in         : device float [batch][n_vn]: observations y if sigma != NULL
  *                (LLR = 2y/sigma^2 formed on the device), else channel LLRs.
@@ -399,7 +402,8 @@ typedef struct mld_plan mld_plan;
 int mld_plan_create(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan **out);
 /* Enqueue the plan's CUDA graph on `stream` (one launch). */
 int mld_plan_launch(mld_plan *p, void *stream);
-/* Number of kernel launches inside the plan's graph. */
+/* Number of kernel launches inside the plan's graph (with early termination
+ * the loop's body, two iterations, counts once). */
 int mld_plan_stats(const mld_plan *p, int64_t *launches);
 int mld_plan_destroy(mld_plan *p);
 /* Create a plan, launch it on `stream`, wait for the stream, destroy it. */

@@ -29,6 +29,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
     float *const accbuf[3] = {d->Lv, d->Lv2, d->Lv3};
     auto acc_of = [&](int32_t l) { return accbuf[(iters - l) % 3]; };
 
+    const int32_t cap_iters = iters;
     d->sample_now = true;
     InArgs ia{in, sigma, g->unit, h.n_vn, h.n_core, h.n_deg1, batch, d->lmax, d->scale_in, d->lmax_i, d->amin_i,
               d->lch, acc_mode ? acc_of(0) : d->Lv, d->lch1, d->post1, d->phi1};
@@ -103,7 +104,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
         }
         return timed_launch(d, kClsSyn, st, "k_lane_update", [&] {
             k_lane_update<W><<<lane_blocks, 128, 0, st>>>(d->done, d->fail, d->iters, d->conv, batch, l,
-                                                           et_mode ? 1 : 0);
+                                                           cap_iters, et_mode ? 1 : 0);
         });
     };
 
@@ -330,7 +331,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
         if (ca.fuse) {  // codewords whose iteration l-1 satisfied every check stop there
             int s = timed_launch(d, kClsSyn, st, "k_lane_update", [&] {
                 k_lane_update<W><<<lane_blocks, 128, 0, st>>>(d->done, ca.fail_prev, d->iters, d->conv, batch,
-                                                               l - 1, 1);
+                                                               l - 1, cap_iters, 1);
             });
             if (s != MLD_OK) return s;
         }
@@ -375,7 +376,7 @@ template <typename MsgT>
 int dispatch_w(mld_decoder *d, const float *in, const float *sigma, const uint8_t *syn, int32_t batch,
                int32_t iters, bool et, uint8_t *bits, float *post, uint8_t *conv, int32_t *it,
                cudaStream_t st, bool out_dev) {
-    switch (d->W) {
+    switch (decode_width(d, batch)) {
         case 8: return run_decode<MsgT, 8>(d, in, sigma, syn, batch, iters, et, bits, post, conv, it, st, out_dev);
         case 16: return run_decode<MsgT, 16>(d, in, sigma, syn, batch, iters, et, bits, post, conv, it, st, out_dev);
         case 32: return run_decode<MsgT, 32>(d, in, sigma, syn, batch, iters, et, bits, post, conv, it, st, out_dev);

@@ -405,6 +405,10 @@ int mld_decoder_create(const mld_graph *g, const mld_opts *opts, mld_decoder **o
     d->device = g->device;
     d->msg = opts->msg_dtype;
     d->W = W;
+    // the kernels of these options exist at the default width only
+    d->narrow_ok = opts->slab_width == 0 && opts->vn_update == MLD_VN_GATHER &&
+                   opts->schedule == MLD_SCHED_FLOODING && opts->check_rule == MLD_CHECK_SUM_PRODUCT &&
+                   opts->staging == MLD_STAGE_DIRECT;
     d->vn_update = opts->vn_update;
     d->schedule = opts->schedule;
     d->check_rule = opts->check_rule;
@@ -684,6 +688,7 @@ extern "C" int mld_decode_noalloc(const mld_graph *g, int32_t msg_dtype, const f
     d.device = g->device;
     d.msg = msg_dtype;
     d.W = W;
+    d.narrow_ok = true;
     d.max_batch = batch;
     d.max_slabs = slabs;
     set_units(&d, 25.f);

@@ -1812,10 +1812,20 @@ __global__ void __launch_bounds__(kBlock) k_syndrome_check(SynArgs a) {
                      static_cast<int64_t>(gridDim.x) * blockDim.x, slab);
 }
 
-// per-codeword bookkeeping after a syndrome check at iteration l
+// Lanes past the batch in word i of a slab's done words (widths up to 64).
+__host__ __device__ inline uint32_t padding_lanes(int32_t batch, int W, int slab, int i) {
+    const int wb = W >= 32 ? 32 : W;  // lanes per word
+    const uint32_t full = W >= 32 ? 0xFFFFFFFFu : ((1u << W) - 1u);
+    const int real = batch - slab * W - i * 32;
+    return real <= 0 ? full : (real >= wb ? 0u : (full & ~((1u << real) - 1u)));
+}
+
+// per-codeword bookkeeping after a syndrome check at iteration l: with early
+// termination a codeword stops at its syndrome match or at the cap, with the
+// outputs of that iteration
 template <int W>
 __device__ __forceinline__ void lane_body(uint32_t *done, const uint32_t *fail, int32_t *iters,
-                                          uint8_t *conv, int32_t batch, int32_t l, int et, int b) {
+                                          uint8_t *conv, int32_t batch, int32_t l, int32_t cap, int et, int b) {
     constexpr int DW = (W + 31) / 32;
     if (b >= batch) return;
     const int slab = b / W, w = b % W;
@@ -1823,10 +1833,10 @@ __device__ __forceinline__ void lane_body(uint32_t *done, const uint32_t *fail, 
     const uint32_t bit = 1u << (w & 31);
     const bool ok = (fail[word] & bit) == 0u;
     if (et) {
-        if (done[word] & bit) return;  // frozen at an earlier iteration
+        if (done[word] & bit) return;  // stopped at an earlier iteration
         iters[b] = l;
         conv[b] = ok ? 1 : 0;
-        if (ok) atomicOr(done + word, bit);
+        if (ok || l >= cap) atomicOr(done + word, bit);
     } else {
         iters[b] = l;
         conv[b] = ok ? 1 : 0;
@@ -1835,8 +1845,8 @@ __device__ __forceinline__ void lane_body(uint32_t *done, const uint32_t *fail, 
 
 template <int W>
 __global__ void k_lane_update(uint32_t *done, const uint32_t *fail, int32_t *iters,
-                              uint8_t *conv, int32_t batch, int32_t l, int et) {
-    lane_body<W>(done, fail, iters, conv, batch, l, et, blockIdx.x * blockDim.x + threadIdx.x);
+                              uint8_t *conv, int32_t batch, int32_t l, int32_t cap, int et) {
+    lane_body<W>(done, fail, iters, conv, batch, l, cap, et, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1851,17 +1861,12 @@ __global__ void k_lane_update(uint32_t *done, const uint32_t *fail, int32_t *ite
 template <int W>
 __global__ void k_loop_init(uint32_t *done, int32_t slabs, int32_t batch, int32_t *lctr, int32_t max_iters) {
     constexpr int DW = (W + 31) / 32;
-    constexpr int WB = W >= 32 ? 32 : W;  // lanes per done word
-    constexpr uint32_t full = W >= 32 ? 0xFFFFFFFFu : ((1u << W) - 1u);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) {
         lctr[0] = 0;
         lctr[1] = max_iters;
     }
-    if (i < slabs * DW) {
-        const int real = batch - (i / DW) * W - (i % DW) * 32;  // real lanes in this word
-        done[i] = real <= 0 ? full : (real >= WB ? 0u : (full & ~((1u << real) - 1u)));
-    }
+    if (i < slabs * DW) done[i] = padding_lanes(batch, W, i / DW, i % DW);
 }
 
 // Bookkeeping of iteration l = lctr[0] + off after its syndrome check (fail):
@@ -1871,19 +1876,9 @@ __global__ void k_loop_init(uint32_t *done, int32_t slabs, int32_t batch, int32_
 template <int W>
 __global__ void k_lane_update_dev(uint32_t *done, const uint32_t *fail, uint32_t *fail_next, int32_t nwords,
                                   int32_t *iters, uint8_t *conv, int32_t batch, const int32_t *lctr, int32_t off) {
-    constexpr int DW = (W + 31) / 32;
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < nwords) fail_next[b] = 0u;
-    if (b >= batch) return;
-    const int32_t l = lctr[0] + off;
-    const int slab = b / W, w = b % W;
-    const int word = slab * DW + w / 32;
-    const uint32_t bit = 1u << (w & 31);
-    if (done[word] & bit) return;  // stopped at an earlier iteration
-    const bool ok = (fail[word] & bit) == 0u;
-    iters[b] = l;
-    conv[b] = ok ? 1 : 0;
-    if (ok || l >= lctr[1]) atomicOr(done + word, bit);
+    lane_body<W>(done, fail, iters, conv, batch, lctr[0] + off, lctr[1], 1, b);
 }
 
 // One warp: continue while some lane still iterates, counting the body's two
@@ -2203,7 +2198,8 @@ struct mld_decoder {
     const mld_graph *g = nullptr;
     int device = 0;
     int msg = MLD_MSG_F32;
-    int W = 32;
+    int W = 32;             // slab width the buffers are sized for
+    bool narrow_ok = false; // decode_width may choose a narrower slab
     int max_batch = 0;
     int max_slabs = 0;
     float lmax = 25.f, amin = 0.f;   // LLR clamp and phi(lmax), nats
@@ -2269,6 +2265,22 @@ void tape_release(mld_decoder *d);
 }  // namespace mld
 
 namespace {
+
+// Slab width of a call with `batch` codewords.  A batch that does not fill the
+// decoder's (default) slab runs in the narrowest slab that holds it: the
+// arithmetic and, down to 32-byte rows, the bytes of the lanes past the batch
+// are saved, at a higher cost per lane (rate 0.1, 64 codewords, half, widths
+// 64 / 32 / 16 / 8: n = 65536 37 / 42 / 46 / 53 us an iteration, n = 10^6 404
+// / 479 / 618 / 863 us; so 16 codewords at n = 10^6 take 155 us in a slab of
+// 16 and 404 us in one of 64).  Batches of several slabs keep the full width:
+// splitting their last one saves lanes but not their price.  A codeword's
+// arithmetic does not depend on the width.
+inline int decode_width(const mld_decoder *d, int32_t batch) {
+    if (!d->narrow_ok) return d->W;
+    int w = d->W;
+    while (w > 8 && batch <= w / 2) w /= 2;
+    return w;
+}
 
 // Sets the clamps and the nats <-> bits scales of a decoder from its lmax.
 inline void set_units(mld_decoder *d, float lmax) {

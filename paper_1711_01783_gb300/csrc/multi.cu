@@ -1,7 +1,9 @@
 // Uneven batches: many codewords over several Tanner graphs (different
 // rates and lengths), each group with its own iteration cap, decoded by one
 // schedule of launches that is captured once into a CUDA graph and replayed
-// with a single launch.
+// with a single launch.  With early termination the iterations are the body of
+// a conditional loop inside that graph, run by the device until every codeword
+// has stopped.
 //
 // The paper decodes a batch of codewords of one code with a fixed number of
 // iterations (Results, "High speed error correction with MET-LDPC codes";
@@ -9,7 +11,9 @@
 // jobs that share its kernel shape: a device table of segments (job, block
 // range) tells each block which job, slab and check class it serves.  With
 // early termination (Methods, Step 5) each codeword stops at its first
-// syndrome match; its slab is skipped once all its codewords have stopped.
+// syndrome match or at its job's cap; its slab is skipped once all its
+// codewords have stopped, and lanes past the batch count as stopped from the
+// start.
 #include <map>
 #include <tuple>
 
@@ -30,7 +34,7 @@ struct JobDev {
     uint32_t *done, *fail;   // fail: two buffers of slabs*DW words (iteration parity)
     int32_t *iters;
     uint8_t *conv;
-    int32_t n_vn, n_cn, batch, slabs, W;
+    int32_t n_vn, n_cn, batch, slabs, W, max_iters;
 };
 
 // One job's share of a launch: blocks block0 .. block0 + bps*slabs - 1.
@@ -45,42 +49,35 @@ __device__ __forceinline__ int find_seg(const Seg *segs, int nseg) {
     return k;
 }
 
-// Check arguments of job j at iteration l: the degree-1 decision buffer of
-// l's parity, and for the fused syndrome check (seg flag 2, l >= 2) the
-// buffers of iteration l-1.
+// Check arguments of job j in an iteration of the given parity (its degree-1
+// decision buffer).
 template <int W>
-__device__ __forceinline__ CnArgs job_cn(const JobDev &j, const Seg &sg, int32_t l) {
-    constexpr int DW = (W + 31) / 32;
+__device__ __forceinline__ CnArgs job_cn(const JobDev &j, const Seg &sg, int parity) {
     CnArgs a = j.cn;
     a.final_pass = sg.flags & 1;
-    const size_t h1 = static_cast<size_t>(j.slabs) * a.n_deg1 * (W / 8);
-    a.hb1 = j.cn.hb1 + static_cast<size_t>(l & 1) * h1;
-    a.hb1_prev = j.cn.hb1 + static_cast<size_t>((l - 1) & 1) * h1;
-    a.fail_prev = j.fail + static_cast<size_t>((l - 1) & 1) * j.slabs * DW;
-    a.fuse = ((sg.flags & 2) && l >= 2) ? 1 : 0;
+    a.hb1 = j.cn.hb1 + static_cast<size_t>(parity) * j.slabs * a.n_deg1 * (W / 8);
     return a;
 }
 
-// The decisions-only form carries the fused syndrome.
 template <typename MsgT, int W, int DC, int DD, int PASS>
 __global__ void __launch_bounds__(kBlock, (kCheckBlocksPerSm<DC + DD>))
-    km_check(const JobDev *jobs, const Seg *segs, int nseg, int32_t l) {
+    km_check(const JobDev *jobs, const Seg *segs, int nseg, int parity) {
     const Seg sg = segs[find_seg(segs, nseg)];
-    const CnArgs a = job_cn<W>(jobs[sg.job], sg, l);
+    const CnArgs a = job_cn<W>(jobs[sg.job], sg, parity);
     const int local = blockIdx.x - sg.block0;
     const int slab = local / sg.bps;
     if (a.et && slab_all_done<W>(a.done, slab)) return;
     // the segment's grid is capped for register classes (build_plan)
     extern __shared__ __align__(128) unsigned char smem[];
-    check_class_body<MsgT, W, DC, DD, PASS, false, PASS == kPassHard>(
+    check_class_body<MsgT, W, DC, DD, PASS>(
         a, sg.cl, static_cast<int64_t>(local % sg.bps) * blockDim.x + threadIdx.x, sg.bps, slab, smem);
 }
 
 template <typename MsgT, int W>
 __global__ void __launch_bounds__(kBlock) km_check_irregular(const JobDev *jobs, const Seg *segs, int nseg,
-                                                             int32_t l) {
+                                                             int parity) {
     const Seg sg = segs[find_seg(segs, nseg)];
-    const CnArgs a = job_cn<W>(jobs[sg.job], sg, l);
+    const CnArgs a = job_cn<W>(jobs[sg.job], sg, parity);
     const int local = blockIdx.x - sg.block0;
     const int slab = local / sg.bps;
     if (a.et && slab_all_done<W>(a.done, slab)) return;
@@ -114,16 +111,48 @@ __global__ void __launch_bounds__(kBlock) km_syndrome(const JobDev *jobs, const 
                      static_cast<int64_t>(sg.bps) * blockDim.x, slab);
 }
 
-// Reads this iteration's fail words and clears the other buffer for the next.
+// Bookkeeping of iteration l (+ lctr[0] inside the loop) after its syndrome
+// check: reads this iteration's fail words and clears the other buffer for the
+// next.  With early termination a codeword stops at its syndrome match or at
+// its job's cap.
 template <int W>
 __global__ void __launch_bounds__(kBlock) km_lane(const JobDev *jobs, const Seg *segs, int nseg, int32_t l,
-                                                  int parity) {
+                                                  int parity, const int32_t *lctr) {
     constexpr int DW = (W + 31) / 32;
     const Seg sg = segs[find_seg(segs, nseg)];
     const JobDev &j = jobs[sg.job];
     const int t = (blockIdx.x - sg.block0) * blockDim.x + threadIdx.x;
-    lane_body<W>(j.done, j.fail + parity * j.slabs * DW, j.iters, j.conv, j.batch, l, j.cn.et, t);
+    if (lctr) l += lctr[0];
+    lane_body<W>(j.done, j.fail + parity * j.slabs * DW, j.iters, j.conv, j.batch, l, j.max_iters, j.cn.et, t);
     if (t < j.slabs * DW) j.fail[(1 - parity) * j.slabs * DW + t] = 0u;
+}
+
+// Lane words of every job at the start: padding lanes count as stopped, no
+// failures yet; the loop's iteration counter at 0.  One block per job.
+__global__ void __launch_bounds__(kBlock) km_init(const JobDev *jobs, int32_t *lctr) {
+    const JobDev &j = jobs[blockIdx.x];
+    const int dw = (j.W + 31) / 32;
+    for (int i = threadIdx.x; i < j.slabs * dw; i += blockDim.x)
+        j.done[i] = padding_lanes(j.batch, j.W, i / dw, i % dw);
+    for (int i = threadIdx.x; i < 2 * j.slabs * dw; i += blockDim.x) j.fail[i] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *lctr = 0;
+}
+
+// Continue while some lane of some job still iterates, counting the body's two
+// iterations (one block).
+__global__ void __launch_bounds__(kBlock) km_loop_cond(const JobDev *jobs, int n_jobs, int32_t *lctr,
+                                                       cudaGraphConditionalHandle h) {
+    bool all = true;
+    for (int k = 0; k < n_jobs; ++k) {
+        const JobDev &j = jobs[k];
+        const uint32_t full = j.W >= 32 ? 0xFFFFFFFFu : ((1u << j.W) - 1u);
+        for (int i = threadIdx.x; i < j.slabs * ((j.W + 31) / 32); i += blockDim.x) all = all && j.done[i] == full;
+    }
+    all = __syncthreads_and(all);
+    if (threadIdx.x == 0) {
+        if (!all) *lctr += 2;
+        cudaGraphSetConditional(h, all ? 0u : 1u);
+    }
 }
 
 template <int W, int F>
@@ -151,12 +180,13 @@ __global__ void __launch_bounds__(kBlock) km_deinterleave(const JobDev *jobs, co
 // ---------------------------------------------------------------------------
 // schedule
 // ---------------------------------------------------------------------------
-enum OpKind { kOpMemset, kOpInterleave, kOpSynIn, kOpHard, kOpCheck, kOpVar, kOpSyn, kOpLane, kOpOut };
+enum OpKind { kOpMemset, kOpInit, kOpInterleave, kOpSynIn, kOpHard, kOpCheck, kOpVar, kOpSyn, kOpLane, kOpOut };
 
 struct Op {
     int kind = 0, half = 0, W = 0, dc = 0, dd = 0, parity = 0;
     int pass = 0;  // check ops: kPass*
     int32_t l = 0;
+    bool in_loop = false;  // l counts from the loop's iteration counter
     int seg0 = 0, nseg = 0, blocks = 0;
     // memset / hard-decision ops
     void *ptr = nullptr;
@@ -173,7 +203,11 @@ struct mld_plan {
     int device = 0;
     JobDev *d_jobs = nullptr;
     Seg *d_segs = nullptr;
-    std::vector<Op> ops;
+    int32_t *d_lctr = nullptr;  // iterations before the loop's current body
+    int n_jobs = 0;
+    // the schedule: before, one body of the early-termination loop (empty
+    // without one), after
+    std::vector<Op> before, body, after;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -193,11 +227,11 @@ void launch_check_op(const mld_plan *p, const Op &op, cudaStream_t st) {
         else if (op.pass == kPassPlain) allow_smem<sm>(km_check<MsgT, W, DCV, DDV, kPassPlain>);    \
         else allow_smem<sm>(km_check<MsgT, W, DCV, DDV, kPassFull>);                                \
         if (op.pass == kPassHard)                                                                   \
-            km_check<MsgT, W, DCV, DDV, kPassHard><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.l); \
+            km_check<MsgT, W, DCV, DDV, kPassHard><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.parity); \
         else if (op.pass == kPassPlain)                                                             \
-            km_check<MsgT, W, DCV, DDV, kPassPlain><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.l); \
+            km_check<MsgT, W, DCV, DDV, kPassPlain><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.parity); \
         else                                                                                        \
-            km_check<MsgT, W, DCV, DDV, kPassFull><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.l); \
+            km_check<MsgT, W, DCV, DDV, kPassFull><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.parity); \
         return;                                                                                     \
     }
     MLD_CASE(1, 0) MLD_CASE(2, 0) MLD_CASE(3, 0) MLD_CASE(4, 0)
@@ -205,7 +239,7 @@ void launch_check_op(const mld_plan *p, const Op &op, cudaStream_t st) {
     MLD_CASE(0, 1) MLD_CASE(1, 1) MLD_CASE(2, 1) MLD_CASE(3, 1)
     MLD_CASE(4, 1) MLD_CASE(5, 1) MLD_CASE(6, 1) MLD_CASE(7, 1)
 #undef MLD_CASE
-    km_check_irregular<MsgT, W><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg, op.l);
+    km_check_irregular<MsgT, W><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg, op.parity);
 }
 
 template <int W>
@@ -231,16 +265,22 @@ void launch_op_w(const mld_plan *p, const Op &op, cudaStream_t st) {
             else km_var<float, W><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg);
             break;
         case kOpSyn: km_syndrome<W><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg, op.parity); break;
-        case kOpLane: km_lane<W><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg, op.l, op.parity); break;
+        case kOpLane: km_lane<W><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg, op.l, op.parity, op.in_loop ? p->d_lctr : nullptr);
+            break;
         case kOpOut: km_deinterleave<W><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg); break;
         default: break;
     }
 }
 
-int enqueue(const mld_plan *p, cudaStream_t st) {
-    for (const Op &op : p->ops) {
+int enqueue(const mld_plan *p, const std::vector<Op> &ops, cudaStream_t st) {
+    for (const Op &op : ops) {
         if (op.kind == kOpMemset) {
             MLD_CUDA(cudaMemsetAsync(op.ptr, 0, op.bytes, st));
+            continue;
+        }
+        if (op.kind == kOpInit) {
+            km_init<<<p->n_jobs, kBlock, 0, st>>>(p->d_jobs, p->d_lctr);
+            MLD_LAUNCHED("km_init");
             continue;
         }
         switch (op.W) {
@@ -254,12 +294,69 @@ int enqueue(const mld_plan *p, cudaStream_t st) {
     return MLD_OK;
 }
 
+// Captures `fill` (work enqueued on the stream it is given) into graph g.
+template <typename F>
+int capture_into(cudaGraph_t g, cudaStream_t cs, F &&fill) {
+    MLD_CUDA(cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    const int s = fill(cs);
+    cudaGraph_t got = nullptr;
+    const cudaError_t e = cudaStreamEndCapture(cs, &got);
+    if (s != MLD_OK) return s;
+    if (e != cudaSuccess) return cuda_fail(e, "plan: capture");
+    return MLD_OK;
+}
+
+// The plan's graph: the ops before the loop, the loop (a conditional node
+// whose body graph holds two iterations), the ops after it.
+int build_graph(mld_plan *p, cudaStream_t cs) {
+    MLD_CUDA(cudaGraphCreate(&p->graph, 0));
+    cudaGraphNode_t last = nullptr;
+    auto add_ops = [&](const std::vector<Op> &ops) -> int {
+        if (ops.empty()) return MLD_OK;
+        cudaGraph_t part = nullptr;
+        MLD_CUDA(cudaGraphCreate(&part, 0));
+        int s = capture_into(part, cs, [&](cudaStream_t st) { return enqueue(p, ops, st); });
+        if (s == MLD_OK) {
+            cudaGraphNode_t node = nullptr;
+            const cudaError_t e = cudaGraphAddChildGraphNode(&node, p->graph, last ? &last : nullptr, last ? 1 : 0, part);
+            if (e != cudaSuccess) s = cuda_fail(e, "plan: child graph");
+            last = node;
+        }
+        cudaGraphDestroy(part);
+        return s;
+    };
+    int s = add_ops(p->before);
+    if (s != MLD_OK) return s;
+    if (!p->body.empty()) {
+        cudaGraphConditionalHandle h;
+        MLD_CUDA(cudaGraphConditionalHandleCreate(&h, p->graph, 1, cudaGraphCondAssignDefault));
+        cudaGraphNodeParams np{};
+        np.type = cudaGraphNodeTypeConditional;
+        np.conditional.handle = h;
+        np.conditional.type = cudaGraphCondTypeWhile;
+        np.conditional.size = 1;
+        cudaGraphNode_t node = nullptr;
+        MLD_CUDA(cudaGraphAddNode(&node, p->graph, &last, nullptr, 1, &np));
+        last = node;
+        s = capture_into(np.conditional.phGraph_out[0], cs, [&](cudaStream_t st) -> int {
+            const int q = enqueue(p, p->body, st);
+            if (q != MLD_OK) return q;
+            km_loop_cond<<<1, kBlock, 0, st>>>(p->d_jobs, p->n_jobs, p->d_lctr, h);
+            MLD_LAUNCHED("km_loop_cond");
+            return MLD_OK;
+        });
+        if (s != MLD_OK) return s;
+    }
+    return add_ops(p->after);
+}
+
 void plan_free(mld_plan *p) {
     if (!p) return;
     if (p->exec) cudaGraphExecDestroy(p->exec);
     if (p->graph) cudaGraphDestroy(p->graph);
     dfree(p->d_jobs);
     dfree(p->d_segs);
+    dfree(p->d_lctr);
     delete p;
 }
 
@@ -274,7 +371,7 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
         const mld_job &jb = jobs[j];
         mld_decoder *d = jb.decoder;
         const mld::HostGraph &h = d->g->h;
-        const int W = d->W;
+        const int W = decode_width(d, jb.batch);
         const int slabs = (jb.batch + W - 1) / W;
         JobDev x{};
         const bool y_mode = jb.sigma != nullptr;
@@ -302,11 +399,15 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
         x.batch = jb.batch;
         x.slabs = slabs;
         x.W = W;
+        x.max_iters = jb.max_iters;
         jd.push_back(x);
         lmax_iters = std::max(lmax_iters, jb.max_iters);
     }
 
-    // one op per group key; segments of the group are the jobs' shares
+    // one op per group key; segments of the group are the jobs' shares; ops
+    // are appended to the part of the schedule being built
+    std::vector<Op> *ops = &p->before;
+    bool in_loop = false;
     using Key = std::tuple<int, int, int, int, int, int>;  // kind, half, W, dc, dd, pass
     auto flush = [&](std::map<Key, std::vector<Seg>> &groups, int32_t l, int parity) {
         for (auto &kv : groups) {
@@ -318,6 +419,7 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
             op.dd = std::get<4>(kv.first);
             op.pass = std::get<5>(kv.first);
             op.l = l;
+            op.in_loop = in_loop;
             op.parity = parity;
             op.seg0 = static_cast<int>(segs.size());
             op.nseg = static_cast<int>(kv.second.size());
@@ -328,7 +430,7 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
                 segs.push_back(s);
             }
             op.blocks = b0;
-            if (op.blocks > 0) p->ops.push_back(op);
+            if (op.blocks > 0) ops->push_back(op);
             else segs.resize(op.seg0);
         }
         groups.clear();
@@ -346,43 +448,38 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
     // prologue: clear messages and per-codeword state, interleave inputs
     for (int32_t j = 0; j < n_jobs; ++j) {
         const mld_decoder *d = jobs[j].decoder;
-        const mld::HostGraph &h = d->g->h;
         const size_t msz = d->msg == MLD_MSG_F16 ? 2 : 4;
-        const size_t DW = (d->W + 31) / 32;
         Op m;
         m.kind = kOpMemset;
         m.ptr = d->r;
-        m.bytes = static_cast<size_t>(jd[j].slabs) * h.e_core * d->W * msz;
-        if (m.bytes) p->ops.push_back(m);
-        m.ptr = d->done;
-        m.bytes = sizeof(uint32_t) * jd[j].slabs * DW;
-        p->ops.push_back(m);
-        m.ptr = d->fail;
-        m.bytes = 2 * sizeof(uint32_t) * jd[j].slabs * DW;
-        p->ops.push_back(m);
+        m.bytes = static_cast<size_t>(jd[j].slabs) * d->g->h.e_core * jd[j].W * msz;
+        if (m.bytes) ops->push_back(m);
+    }
+    if (n_jobs > 0) {
+        Op m;
+        m.kind = kOpInit;
+        ops->push_back(m);
     }
     for (int32_t j = 0; j < n_jobs; ++j) {
         const mld_decoder *d = jobs[j].decoder;
         const int half = d->msg == MLD_MSG_F16;
         if (jd[j].n_vn > 0)
-            groups[Key{kOpInterleave, half, d->W, 0, 0, 0}].push_back(seg(j, (jd[j].n_vn + 31) / 32, jd[j].slabs, 0));
+            groups[Key{kOpInterleave, half, jd[j].W, 0, 0, 0}].push_back(seg(j, (jd[j].n_vn + 31) / 32, jd[j].slabs, 0));
         if (jd[j].n_cn > 0)
-            groups[Key{kOpSynIn, 0, d->W, 0, 0, 0}].push_back(seg(j, (jd[j].n_cn + 31) / 32, jd[j].slabs, 0));
+            groups[Key{kOpSynIn, 0, jd[j].W, 0, 0, 0}].push_back(seg(j, (jd[j].n_cn + 31) / 32, jd[j].slabs, 0));
     }
     flush(groups, 0, 0);
 
     auto syndrome_round = [&](const std::vector<int32_t> &js, int32_t l) {
         const int parity = l & 1;
         for (int32_t j : js) {
-            const mld_decoder *d = jobs[j].decoder;
             const int bps = syndrome_blocks(jd[j].n_cn, sm_count);
-            if (jd[j].n_cn > 0) groups[Key{kOpSyn, 0, d->W, 0, 0, 0}].push_back(seg(j, bps, jd[j].slabs, 0));
+            if (jd[j].n_cn > 0) groups[Key{kOpSyn, 0, jd[j].W, 0, 0, 0}].push_back(seg(j, bps, jd[j].slabs, 0));
         }
         flush(groups, l, parity);
         for (int32_t j : js) {
-            const mld_decoder *d = jobs[j].decoder;
-            const int lanes = std::max(jd[j].batch, jd[j].slabs * ((d->W + 31) / 32));
-            groups[Key{kOpLane, 0, d->W, 0, 0, 0}].push_back(seg(j, (lanes + kBlock - 1) / kBlock, 1, 0));
+            const int lanes = std::max(jd[j].batch, jd[j].slabs * ((jd[j].W + 31) / 32));
+            groups[Key{kOpLane, 0, jd[j].W, 0, 0, 0}].push_back(seg(j, (lanes + kBlock - 1) / kBlock, 1, 0));
         }
         flush(groups, l, parity);
     };
@@ -396,76 +493,80 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
             const mld::HostGraph &h = d->g->h;
             Op op;
             op.kind = kOpHard;
-            op.W = d->W;
+            op.W = jd[j].W;
             op.slabs = jd[j].slabs;
             if (h.n_core > 0) {
                 op.post = d->Lv;
                 op.count = h.n_core;
                 op.hb = d->hb_core;
-                p->ops.push_back(op);
+                ops->push_back(op);
             }
             if (h.n_deg1 > 0) {
                 op.post = d->post1;
                 op.count = h.n_deg1;
                 op.hb = d->hb1;
-                p->ops.push_back(op);
+                ops->push_back(op);
             }
             zero.push_back(j);
         }
         if (!zero.empty()) syndrome_round(zero, 0);
     }
 
-    // early termination without soft output: degree-1 decisions only, and for
-    // graphs whose checks are all in register classes the syndrome of
-    // iteration l-1 is formed inside check pass l (then only the last
-    // iteration gets a separate syndrome check)
-    auto hard1_job = [&](int32_t j) { return et && !jobs[j].post_out; };
-    auto fused_job = [&](int32_t j) { return hard1_job(j) && jobs[j].decoder->g->fusable; };
-    for (int32_t l = 1; l <= lmax_iters; ++l) {
-        std::vector<int32_t> active, checked, lanes;
-        for (int32_t j = 0; j < n_jobs; ++j)
-            if (jobs[j].max_iters >= l) active.push_back(j);
+    // iteration l (counted from the loop's counter inside the loop) of the
+    // given jobs; `last_of(j)`: also form decisions and check the syndrome
+    auto iteration = [&](const std::vector<int32_t> &active, int32_t l, auto &&last_of) {
+        const int parity = l & 1;
+        std::vector<int32_t> checked;
         for (int32_t j : active) {
             const mld_decoder *d = jobs[j].decoder;
             const int half = d->msg == MLD_MSG_F16;
-            const int fl = ((et || l == jobs[j].max_iters) ? 1 : 0) | (fused_job(j) ? 2 : 0);
-            for (const ClassLaunch &cl : d->g->launches[width_index(d->W)]) {
+            const int fl = last_of(j) ? 1 : 0;
+            for (const ClassLaunch &cl : d->g->launches[width_index(jd[j].W)]) {
                 const int dd = cl.deg - cl.dc;
                 const bool regular = cl.dc >= 0 && (dd == 0 || dd == 1);
-                const int pass = !regular ? kPassFull : hard1_job(j) ? kPassHard : (fl & 1) ? kPassFull : kPassPlain;
+                // early termination without soft output: degree-1 decisions only
+                const int pass = !regular ? kPassFull : (et && !jobs[j].post_out) ? kPassHard : fl ? kPassFull : kPassPlain;
                 Seg s = seg(j, regular ? class_blocks(cl, sm_count) : cl.blocks, jd[j].slabs, fl);
                 s.cl = cl;
-                groups[Key{kOpCheck, half, d->W, regular ? cl.dc : -1, regular ? dd : -1, pass}].push_back(s);
+                groups[Key{kOpCheck, half, jd[j].W, regular ? cl.dc : -1, regular ? dd : -1, pass}].push_back(s);
             }
-            if (fused_job(j) && l >= 2) lanes.push_back(j);
         }
-        flush(groups, l, 0);
-        // the codewords of fused jobs whose iteration l-1 satisfied every check
-        // stop there (the lane op also clears the other fail buffer)
-        if (!lanes.empty()) {
-            for (int32_t j : lanes) {
-                const mld_decoder *d = jobs[j].decoder;
-                const int nl = std::max(jd[j].batch, jd[j].slabs * ((d->W + 31) / 32));
-                groups[Key{kOpLane, 0, d->W, 0, 0, 0}].push_back(seg(j, (nl + kBlock - 1) / kBlock, 1, 0));
-            }
-            flush(groups, l - 1, (l - 1) & 1);
-        }
+        flush(groups, l, parity);
         for (int32_t j : active) {
             const mld_decoder *d = jobs[j].decoder;
-            const int half = d->msg == MLD_MSG_F16;
-            const int fl = (et || l == jobs[j].max_iters) ? 1 : 0;
-            const int tpc = d->W / kK;
-            const int bps = grid_x(static_cast<int64_t>(d->g->h.n_core) * tpc);
-            if (d->g->h.n_core > 0) groups[Key{kOpVar, half, d->W, 0, 0, 0}].push_back(seg(j, bps, jd[j].slabs, fl));
-            if (fl && (!fused_job(j) || l == jobs[j].max_iters)) checked.push_back(j);
+            const int bps = grid_x(static_cast<int64_t>(d->g->h.n_core) * (jd[j].W / kK));
+            const int fl = last_of(j) ? 1 : 0;
+            if (d->g->h.n_core > 0)
+                groups[Key{kOpVar, d->msg == MLD_MSG_F16, jd[j].W, 0, 0, 0}].push_back(seg(j, bps, jd[j].slabs, fl));
+            if (fl) checked.push_back(j);
         }
-        flush(groups, l, 0);
+        flush(groups, l, parity);
         if (!checked.empty()) syndrome_round(checked, l);
+    };
+    if (et) {
+        // the device repeats two iterations until every codeword has stopped
+        std::vector<int32_t> active;
+        for (int32_t j = 0; j < n_jobs; ++j)
+            if (jobs[j].max_iters > 0) active.push_back(j);
+        if (!active.empty()) {
+            ops = &p->body;
+            in_loop = true;
+            for (int32_t l = 1; l <= 2; ++l) iteration(active, l, [](int32_t) { return true; });
+            in_loop = false;
+        }
+    } else {
+        for (int32_t l = 1; l <= lmax_iters; ++l) {
+            std::vector<int32_t> active;
+            for (int32_t j = 0; j < n_jobs; ++j)
+                if (jobs[j].max_iters >= l) active.push_back(j);
+            iteration(active, l, [&](int32_t j) { return jobs[j].max_iters == l; });
+        }
     }
+    ops = &p->after;
 
     for (int32_t j = 0; j < n_jobs; ++j)
         if (jd[j].n_vn > 0)
-            groups[Key{kOpOut, 0, jobs[j].decoder->W, 0, 0, 0}].push_back(seg(j, (jd[j].n_vn + 31) / 32, jd[j].slabs, 0));
+            groups[Key{kOpOut, 0, jd[j].W, 0, 0, 0}].push_back(seg(j, (jd[j].n_vn + 31) / 32, jd[j].slabs, 0));
     flush(groups, 0, 0);
     return MLD_OK;
 }
@@ -508,26 +609,19 @@ int mld_plan_create(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_pla
     mld_plan *p = new (std::nothrow) mld_plan();
     if (!p) return mld::fail(MLD_ENOMEM, "plan_create: host allocation");
     p->device = dev;
+    p->n_jobs = n_jobs;
     std::vector<JobDev> jd;
     std::vector<Seg> segs;
     s = build_plan(jobs, n_jobs, flags, p, jd, segs);
     if (s == MLD_OK) s = upload(&p->d_jobs, jd);
     if (s == MLD_OK) s = upload(&p->d_segs, segs);
+    if (s == MLD_OK) s = dalloc(&p->d_lctr, 1);
     cudaStream_t cs = nullptr;
     if (s == MLD_OK) {
         cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
         if (e != cudaSuccess) s = cuda_fail(e, "cudaStreamCreate");
     }
-    if (s == MLD_OK) {
-        cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) s = cuda_fail(e, "cudaStreamBeginCapture");
-        if (s == MLD_OK) {
-            const int es = enqueue(p, cs);
-            e = cudaStreamEndCapture(cs, &p->graph);
-            if (es != MLD_OK) s = es;
-            else if (e != cudaSuccess) s = cuda_fail(e, "cudaStreamEndCapture");
-        }
-    }
+    if (s == MLD_OK) s = build_graph(p, cs);
     if (s == MLD_OK) {
         cudaError_t e = cudaGraphInstantiate(&p->exec, p->graph, 0);
         if (e != cudaSuccess) s = cuda_fail(e, "cudaGraphInstantiate");
@@ -554,7 +648,9 @@ int mld_plan_stats(const mld_plan *p, int64_t *launches) {
     mld::clear_error();
     if (!p || !launches) return mld::fail(MLD_EINVAL, "plan_stats: null pointer");
     int64_t n = 0;
-    for (const Op &op : p->ops) n += (op.kind == kOpMemset) ? 0 : 1;
+    for (const std::vector<Op> *part : {&p->before, &p->body, &p->after})
+        for (const Op &op : *part) n += (op.kind == kOpMemset) ? 0 : 1;
+    if (!p->body.empty()) n += 1;  // the loop's condition
     *launches = n;
     return MLD_OK;
 }
