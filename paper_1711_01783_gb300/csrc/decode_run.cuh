@@ -81,7 +81,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
                 static_cast<int64_t>(launches[big].blocks) * launches[big].deg)
                 big = static_cast<int>(i);
     }
-    const dim3 vn_grid(grid_x(static_cast<int64_t>(h.n_core) * TPC), slabs);
+    const dim3 vn_grid(grid_x(static_cast<int64_t>(h.n_core) * (W / kVnLanes)), slabs);
     int sm_count = 152;
     cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, d->device);
     const dim3 syn_grid(syndrome_blocks(h.n_cn, sm_count), slabs);

@@ -211,19 +211,16 @@ __device__ __forceinline__ uint64_t l2_evict_last() {
 }
 // loads of a row that nothing reads again before the next pass rewrites or
 // displaces it
-__device__ __forceinline__ uint2 load_once(const uint2 *a, uint64_t policy) {
-    uint2 v;
-    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v2.u32 {%0,%1}, [%2], %3;"
-                 : "=r"(v.x), "=r"(v.y)
+__device__ __forceinline__ uint4 load_once(const uint4 *a, uint64_t policy) {
+    uint4 v;
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(a), "l"(policy));
     return v;
 }
 __device__ __forceinline__ float4 load_once(const float4 *a, uint64_t policy) {
-    float4 v;
-    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "l"(a), "l"(policy));
-    return v;
+    const uint4 u = load_once(reinterpret_cast<const uint4 *>(a), policy);
+    return make_float4(bitsf(u.x), bitsf(u.y), bitsf(u.z), bitsf(u.w));
 }
 __device__ __forceinline__ void store_hint(float4 *a, float4 v, uint64_t policy) {
     asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(a), "f"(v.x), "f"(v.y), "f"(v.z),
@@ -827,21 +824,21 @@ __device__ __forceinline__ void check_class_body(const CnArgs &a, const ClassLau
     const int32_t stride = blocks * (kBlock / TPC);
     const uint32_t sm = smem_u32(smem);
     int32_t v[DC > 0 ? DC : 1];  // column indices of the check whose operands are requested next,
-    int32_t cn = 0;              // and its position in the class
+    int32_t cn = 0;              // and (LAY) its position in the class
     uint32_t sbn = 0;            // syndrome byte of the check requested last
     auto cols = [&](int32_t j) {
         j = min(j, cl.count - 1);  // (past the end: a valid address that nothing uses)
 #pragma unroll
         for (int i = 0; i < DC; ++i) v[i] = __ldg(a.col + cl.e0 + j * DC + i);
-        cn = LAY ? __ldg(pos + j) - cl.c0 : j;
+        if constexpr (LAY) cn = __ldg(pos + j) - cl.c0;
     };
     auto request = [&](int32_t j, int slot) {
-        if (j < cl.count) {
+        const int32_t c = LAY ? cn : j;
+        if (j < cl.count)
             Ring::template request<W>(sm + slot * kStage, v, lvb, rb + static_cast<size_t>(j * DC) * W,
-                                      pb + static_cast<size_t>(cn * DD) * W);
-            sbn = sbp[static_cast<size_t>(cn) * NB];
-        }
+                                      pb + static_cast<size_t>(c * DD) * W);
         cp_async_commit();  // (an empty group past the end keeps the count)
+        sbn = sbp[static_cast<size_t>(LAY ? cn : min(j, cl.count - 1)) * NB];
     };
     uint32_t fail = 0;
     int32_t j = static_cast<int32_t>(t0 / TPC);
@@ -851,7 +848,7 @@ __device__ __forceinline__ void check_class_body(const CnArgs &a, const ClassLau
     cols(j + stride);
     for (int slot = 0; j < cl.count; j += stride, slot ^= 1) {
         const uint32_t sb = sbn >> (lane0 & 7);
-        const int32_t s0 = cl.s0 + c * DD;
+        const int32_t s0 = cl.s0 + (LAY ? c : j) * DD;
         request(j + stride, slot ^ 1);
         c = cn;
         cols(j + 2 * stride);
@@ -1647,67 +1644,102 @@ struct VnArgs {
     int want_bits, et;
 };
 
-template <typename MsgT, int W>
+// One thread owns 8 codewords of one VN: 16 bytes of a half row (one load), 32
+// of a float row (two), and one whole byte of decisions.
+constexpr int kVnLanes = 8;
+template <typename MsgT> struct VnRow;
+template <> struct VnRow<__half> {
+    uint4 u;
+    __device__ __forceinline__ void load(const __half *p, uint64_t policy) {
+        u = load_once(reinterpret_cast<const uint4 *>(p), policy);
+    }
+    __device__ __forceinline__ float2 pair(int i) const {
+        const uint32_t w = i == 0 ? u.x : i == 1 ? u.y : i == 2 ? u.z : u.w;
+        return __half22float2(*reinterpret_cast<const __half2 *>(&w));
+    }
+};
+template <> struct VnRow<float> {
+    float4 a, b;
+    __device__ __forceinline__ void load(const float *p, uint64_t policy) {
+        a = load_once(reinterpret_cast<const float4 *>(p), policy);
+        b = load_once(reinterpret_cast<const float4 *>(p + 4), policy);
+    }
+    __device__ __forceinline__ float2 pair(int i) const {
+        return i == 0 ? make_float2(a.x, a.y) : i == 1 ? make_float2(a.z, a.w) : i == 2 ? make_float2(b.x, b.y)
+                                                                                        : make_float2(b.z, b.w);
+    }
+};
+
+// The VN's edges a few per round, every load of a round in flight together;
+// the last round's missing edges are not loaded and add nothing, so the sums
+// are formed in CSC order.  A message row is read once per pass: its lines go
+// past L1 and leave L2 first, so that they do not displace the posteriors,
+// which are stored to stay (the next check pass gathers each row once per
+// edge).  The pass is bound by HBM (each message row once, in the order of a
+// random permutation).  Rate 0.1, n = 10^6, 64 codewords, half, 4 codewords
+// per thread: 0.132 ms with plain loads and stores, 0.120 ms with the
+// priorities, and the check pass 0.285 -> 0.275 ms; 8 codewords per thread
+// at 2 / 4 / 6 / 8 edges per round 0.123 / 0.123 / 0.119 / 0.121 ms (rate 0.02:
+// 0.056 -> 0.052 ms at 6).  Rate 0.05, 32 codewords, float: 0.086 -> 0.078 ms,
+// 8 codewords per thread 0.071 / 0.072 / 0.077 / 0.073 ms.
+template <typename MsgT, int W, int kRound = IsHalf<MsgT>::value ? 6 : 4>
 __device__ __forceinline__ void var_body(const VnArgs &a, int64_t t, int slab) {
-    constexpr int TPC = W / kK;
+    constexpr int TPV = W / kVnLanes;
     constexpr int NB = W / 8;
-    const int32_t v = static_cast<int32_t>(t / TPC);
+    const int32_t v = static_cast<int32_t>(t / TPV);
     if (v >= a.n_core) return;
-    const int lane0 = static_cast<int>(t % TPC) * kK;
+    const int lane0 = static_cast<int>(t % TPV) * kVnLanes;
     const size_t vrow = (static_cast<size_t>(slab) * a.n_core + v) * W + lane0;
     const MsgT *rb = static_cast<const MsgT *>(a.r) + static_cast<size_t>(slab) * a.e_core * W + lane0;
-    float4 acc = ldf4(a.lch + vrow);
+    const float4 l0 = ldf4(a.lch + vrow), l1 = ldf4(a.lch + vrow + 4);
+    float2 acc[4] = {make_float2(l0.x, l0.y), make_float2(l0.z, l0.w), make_float2(l1.x, l1.y), make_float2(l1.z, l1.w)};
     int32_t j = a.vptr[v];
     const int32_t j1 = a.vptr[v + 1];
-    // four edges per round, every load of a round in flight together; the
-    // last round's missing edges are not loaded and add nothing, so the sums
-    // are formed in CSC order (re-reading the round's first row for them, an
-    // L1 hit, needs L1 to hold rows that pass through once).  A message row is
-    // read once per pass: its lines leave L2 first, so that they do not
-    // displace the posteriors.  The pass is bound by HBM (each message row
-    // once, in the order of a random permutation): rate 0.1, n = 10^6, 64
-    // codewords, half 0.132 -> 0.120 ms; rate 0.05, 32 codewords, float 0.087
-    // -> 0.078 ms, and the check pass that gathers the posteriors 0.285 ->
-    // 0.275 ms and 0.148 -> 0.140 ms.  Eight edges per round: 0.130 ms.
-    constexpr int kRound = 4;
-    using Raw = typename Msg<MsgT>::Raw;
     const uint64_t once = l2_evict_first();
     for (; j < j1; j += kRound) {
         const int32_t rem = j1 - j;
         int32_t e[kRound];
-        Raw r[kRound];
+        VnRow<MsgT> r[kRound];
 #pragma unroll
         for (int k = 0; k < kRound; ++k) e[k] = k < rem ? __ldg(a.vedge + j + k) : 0;
 #pragma unroll
         for (int k = 0; k < kRound; ++k)
-            r[k] = k < rem ? load_once(reinterpret_cast<const Raw *>(rb + static_cast<size_t>(e[k]) * W), once) : Raw{};
+            if (k < rem) r[k].load(rb + static_cast<size_t>(e[k]) * W, once);
 #pragma unroll
         for (int k = 0; k < kRound; ++k) {
             if (k < rem) {
-                const float2 p = Msg<MsgT>::pair(r[k], 0), q = Msg<MsgT>::pair(r[k], 1);
-                acc.x += p.x; acc.y += p.y; acc.z += q.x; acc.w += q.y;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[i] = add2(acc[i], r[k].pair(i));
             }
         }
     }
+    float4 o0 = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y), o1 = make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y);
+    float *lv = a.Lv + vrow;
     if (a.et) {
         // converged lanes keep the posterior of their last iteration (with a
         // fused syndrome check a lane is marked after its messages moved on)
-        const uint32_t dn = done_nibble<W>(a.done, slab, lane0);
+        constexpr int DW = (W + 31) / 32;
+        const uint32_t dn = (a.done[slab * DW + lane0 / 32] >> (lane0 & 31)) & 0xFFu;
         if (dn) {
-            const float4 old = *reinterpret_cast<const float4 *>(a.Lv + vrow);
-            if (dn & 1) acc.x = old.x;
-            if (dn & 2) acc.y = old.y;
-            if (dn & 4) acc.z = old.z;
-            if (dn & 8) acc.w = old.w;
+            const float4 p0 = *reinterpret_cast<const float4 *>(lv), p1 = *reinterpret_cast<const float4 *>(lv + 4);
+            if (dn & 1) o0.x = p0.x;
+            if (dn & 2) o0.y = p0.y;
+            if (dn & 4) o0.z = p0.z;
+            if (dn & 8) o0.w = p0.w;
+            if (dn & 16) o1.x = p1.x;
+            if (dn & 32) o1.y = p1.y;
+            if (dn & 64) o1.z = p1.z;
+            if (dn & 128) o1.w = p1.w;
         }
     }
     // the next check pass gathers every posterior row once per edge
-    store_hint(reinterpret_cast<float4 *>(a.Lv + vrow), acc, l2_evict_last());
+    const uint64_t keep = l2_evict_last();
+    store_hint(reinterpret_cast<float4 *>(lv), o0, keep);
+    store_hint(reinterpret_cast<float4 *>(lv + 4), o1, keep);
     if (a.want_bits) {
-        const uint32_t nib = (acc.x < 0.f) | ((acc.y < 0.f) << 1) | ((acc.z < 0.f) << 2) | ((acc.w < 0.f) << 3);
-        const uint32_t other = __shfl_xor_sync(pair_mask(), nib, 1);
-        if ((lane0 & 7) == 0)
-            a.hb[(static_cast<size_t>(slab) * a.n_core + v) * NB + lane0 / 8] = static_cast<uint8_t>(nib | (other << 4));
+        const uint32_t byte = (o0.x < 0.f) | ((o0.y < 0.f) << 1) | ((o0.z < 0.f) << 2) | ((o0.w < 0.f) << 3) |
+                              ((o1.x < 0.f) << 4) | ((o1.y < 0.f) << 5) | ((o1.z < 0.f) << 6) | ((o1.w < 0.f) << 7);
+        a.hb[(static_cast<size_t>(slab) * a.n_core + v) * NB + lane0 / 8] = static_cast<uint8_t>(byte);
     }
 }
 

@@ -534,7 +534,7 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
         flush(groups, l, parity);
         for (int32_t j : active) {
             const mld_decoder *d = jobs[j].decoder;
-            const int bps = grid_x(static_cast<int64_t>(d->g->h.n_core) * (jd[j].W / kK));
+            const int bps = grid_x(static_cast<int64_t>(d->g->h.n_core) * (jd[j].W / kVnLanes));
             const int fl = last_of(j) ? 1 : 0;
             if (d->g->h.n_core > 0)
                 groups[Key{kOpVar, d->msg == MLD_MSG_F16, jd[j].W, 0, 0, 0}].push_back(seg(j, bps, jd[j].slabs, fl));

@@ -506,7 +506,6 @@ template <int W>
 int forward_iters(mld_decoder *d, const WArgs &wa, float *r, float *lv, int t_begin, int t_end, int T, int slabs,
                   cudaStream_t st, mld_tape *tape, float *seg_r, float *seg_lv) {
     const mld::HostGraph &h = d->g->h;
-    constexpr int TPC = W / kK;
     const size_t rsz = static_cast<size_t>(slabs) * h.e_core * W;
     const size_t lsz = static_cast<size_t>(slabs) * h.n_core * W;
     VnArgs va{d->g->vptr, d->g->vedge, h.n_core, h.e_core, r, d->lch, lv, d->hb_core, d->done, 0, 0};
@@ -521,7 +520,7 @@ int forward_iters(mld_decoder *d, const WArgs &wa, float *r, float *lv, int t_be
             MLD_LAUNCHED("kw_check_fwd");
         }
         if (h.n_core > 0) {
-            k_var_update<float, W><<<dim3(grid_x(static_cast<int64_t>(h.n_core) * TPC), slabs), kBlock, 0, st>>>(va);
+            k_var_update<float, W><<<dim3(grid_x(static_cast<int64_t>(h.n_core) * (W / kVnLanes)), slabs), kBlock, 0, st>>>(va);
             MLD_LAUNCHED("k_var_update");
         }
         if (tape && !seg_r && t % tape->k == 0 && t < T)
@@ -607,7 +606,7 @@ int wbp_backward_w(mld_tape *tp, const float *dsoft, float *dw, float *dllr, cud
             }
             if (h.n_core > 0) {
                 VnArgs va{d->g->vptr, d->g->vedge, h.n_core, h.e_core, r, d->lch, d->Lv, d->hb_core, d->done, 0, 0};
-                k_var_update<float, W><<<vgrid, kBlock, 0, s2>>>(va);
+                k_var_update<float, W><<<dim3(grid_x(static_cast<int64_t>(h.n_core) * (W / kVnLanes)), slabs), kBlock, 0, s2>>>(va);
                 MLD_LAUNCHED("k_var_update");
             }
             int s = forward_iters<W>(d, wa, r, d->Lv, t0, t1 - 1, T, slabs, s2, tp, tp->seg_r, tp->seg_lv);
