@@ -18,7 +18,7 @@ BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmetldpc.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["decoder.cu", "decode_f16.cu", "decode_f32.cu", "multi.cu", "wbp.cu", "md.cu", "graph.cpp",
+SOURCES = ["decoder.cu", "decode_f16.cu", "decode_f32.cu", "small_f16.cu", "small_f32.cu", "multi.cu", "wbp.cu", "md.cu", "graph.cpp",
            "ensemble.cpp", "peg.cpp"]
 
 

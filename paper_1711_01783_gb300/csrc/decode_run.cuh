@@ -18,9 +18,6 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
     const int slabs = (batch + W - 1) / W;
     constexpr int TPC = W / kK;
     constexpr int DW = (W + 31) / 32;
-    const size_t rbytes = static_cast<size_t>(slabs) * h.e_core * W * sizeof(MsgT);
-    if (rbytes) MLD_CUDA(cudaMemsetAsync(d->r, 0, rbytes, st));
-    MLD_CUDA(cudaMemsetAsync(d->done, 0, sizeof(uint32_t) * slabs * DW, st));
 
     // Posterior accumulation: iteration l reads the posteriors of l-1 from
     // one of three buffers and adds its messages into the buffer of l,
@@ -33,19 +30,31 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
     d->sample_now = true;
     InArgs ia{in, sigma, g->unit, h.n_vn, h.n_core, h.n_deg1, batch, d->lmax, d->scale_in, d->lmax_i, d->amin_i,
               d->lch, acc_mode ? acc_of(0) : d->Lv, d->lch1, d->post1, d->phi1};
-    if (h.n_vn > 0) {
-        int s = timed_launch(d, kClsLayout, st, "k_interleave_in", [&] {
-            k_interleave_in<W, DecodeFit<MsgT>::value><<<dim3((h.n_vn + 31) / 32, slabs), kBlock, 0, st>>>(ia);
+    const PrologueArgs pa{ia, syn, g->cint, d->sbits, h.n_cn, (h.n_vn + 31) / 32, static_cast<uint4 *>(d->r),
+                          static_cast<size_t>(slabs) * h.e_core * W * sizeof(MsgT) / 16};
+    if (h.n_vn > 0 || h.n_cn > 0) {
+        int s = timed_launch(d, kClsLayout, st, "k_prologue", [&] {
+            k_prologue<W, DecodeFit<MsgT>::value>
+                <<<dim3(pa.in_tiles + (h.n_cn + 31) / 32, slabs), kBlock, 0, st>>>(pa);
         });
         if (s != MLD_OK) return s;
     }
-    if (h.n_cn > 0) {
-        int s = timed_launch(d, kClsLayout, st, "k_syndrome_in", [&] {
-            k_syndrome_in<W><<<dim3((h.n_cn + 31) / 32, slabs), kBlock, 0, st>>>(syn, g->cint, h.n_cn, batch,
-                                                                                d->sbits);
-        });
-        if (s != MLD_OK) return s;
+
+    int sm_count = 152;
+    cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, d->device);
+    // Small problems: every iteration in one launch (not while kernels are
+    // timed one by one).  Its lane results are in d->iters and d->conv, and with
+    // device pointers in the caller's arrays.
+    bool small = false;
+    if (iters > 0 && !d->timing && d->bar && d->schedule == MLD_SCHED_FLOODING &&
+        d->check_rule == MLD_CHECK_SUM_PRODUCT && d->staging == MLD_STAGE_DIRECT && !acc_mode) {
+        const bool hard = et && !post;
+        int32_t *io = out_dev ? iters_out : nullptr;
+        uint8_t *co = out_dev ? conv_out : nullptr;
+        if constexpr (IsHalf<MsgT>::value) small = mld::small_decode_f16(d, W, batch, iters, et, hard, io, co, sm_count, st);
+        else small = mld::small_decode_f32(d, W, batch, iters, et, hard, io, co, sm_count, st);
     }
+    if (!small) MLD_CUDA(cudaMemsetAsync(d->done, 0, sizeof(uint32_t) * slabs * DW, st));
 
     // degree-1 decisions: two buffers, written by iterations of each parity
     // (a codeword's output is read from the one of its last iteration)
@@ -53,19 +62,14 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
     auto hb1_of = [&](int32_t l) { return d->hb1 + static_cast<size_t>(l & 1) * h1; };
     CnArgs ca{g->cptr, g->col, g->dptr, h.n_cn, h.n_core, h.n_deg1, h.e_core,
               d->r, d->Lv, d->lch1, d->phi1, d->post1, d->hb1, d->sbits, d->done,
-              d->lmax_i, d->amin_i, 0, et ? 1 : 0, 0, batch, d->hb1, d->fail};
+              d->lmax_i, d->amin_i, 0, et ? 1 : 0};
     ca.status = d->status;
     ca.stall_test = d->stall_test;
-    // early termination without soft output: degree-1 decisions only, and
-    // the syndrome of iteration l-1 formed inside check pass l (every check
-    // in a register class; otherwise a separate syndrome check per iteration)
     ca.rule = d->check_rule == MLD_CHECK_MIN_SUM ? kRuleMinSum : kRuleSumProduct;
     ca.ms_off = d->ms_off_i;
-    // (the decision-only form is a sum-product property)
+    // early termination without soft output: degree-1 decisions only (a
+    // sum-product property)
     const bool hard1 = et && !post && d->check_rule == MLD_CHECK_SUM_PRODUCT;
-    // the fused syndrome check is for the host-driven loop (decoder views
-    // without a capture stream); otherwise the device loop runs the iterations
-    const bool fused = hard1 && g->fusable && !d->cap;
     VnArgs va{g->vptr, g->vedge, h.n_core, h.e_core, d->r, d->lch, d->Lv, d->hb_core, d->done, 0, et ? 1 : 0};
     SynArgs sa{g->cptr, g->col, g->dptr, h.n_cn, h.n_core, h.n_deg1, d->sbits, d->hb_core, d->hb1,
                d->fail, d->done, et ? 1 : 0, batch};
@@ -82,8 +86,6 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
                 big = static_cast<int>(i);
     }
     const dim3 vn_grid(grid_x(static_cast<int64_t>(h.n_core) * (W / kVnLanes)), slabs);
-    int sm_count = 152;
-    cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, d->device);
     const dim3 syn_grid(syndrome_blocks(h.n_cn, sm_count), slabs);
     // staged check updates: one wave of kStagedBlocksPerSm blocks per SM
     const int staged_cap = d->staging != MLD_STAGE_DIRECT ? sm_count * kStagedBlocksPerSm : 0;
@@ -108,7 +110,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
         });
     };
 
-    if (iters == 0) {
+    if (cap_iters == 0) {
         if (h.n_core > 0) {
             int s = timed_launch(d, kClsLayout, st, "k_hard_bits", [&] {
                 k_hard_bits<W><<<dim3(grid_x(static_cast<int64_t>(h.n_core) * (W / 8)), slabs), kBlock, 0, st>>>(
@@ -130,14 +132,14 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
     // CUDA-graph loop, see k_loop_cond), so no launch follows the iteration at
     // which the last codeword stops.  Decoder views without a capture stream
     // (mld_decode_noalloc) keep the host loop.
-    const bool dev_loop = et && iters > 0 && d->cap && d->lctr && (d->schedule == MLD_SCHED_LAYERED || !fused);
+    if (small) iters = 0;  // the loops below do nothing
+    const bool dev_loop = et && iters > 0 && d->cap && d->lctr;
     if (dev_loop) {
         // one early-terminated iteration of parity `parity` (l odd: 1), whose
         // number is lctr[0] + off, enqueued on stream s
         auto enqueue_half = [&](int parity, int off, cudaStream_t s) -> int {
             CnArgs c2 = ca;
             c2.final_pass = 1;
-            c2.fuse = 0;
             c2.hb1 = d->hb1 + static_cast<size_t>(parity) * h1;
             if (d->schedule == MLD_SCHED_LAYERED) {
                 CnArgs la = c2;
@@ -295,11 +297,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
         const bool last = (l == iters);
         ca.final_pass = (last || et) ? 1 : 0;
         ca.hb1 = hb1_of(l);
-        ca.hb1_prev = hb1_of(l - 1);
-        ca.fail_prev = d->fail + static_cast<size_t>((l - 1) & 1) * slabs * DW;
-        ca.fuse = (fused && l >= 2) ? 1 : 0;
         d->sample_now = ((l - 1) % d->timing_every) == 0;
-        if (ca.fuse) MLD_CUDA(cudaMemsetAsync(ca.fail_prev, 0, sizeof(uint32_t) * slabs * DW, st));
         if (acc_mode && h.n_core > 0) {
             ca.Lv = acc_of(l - 1);
             ca.acc = acc_of(l);
@@ -328,14 +326,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
             }, static_cast<int>(launches.size()));
             if (s != MLD_OK) return s;
         }
-        if (ca.fuse) {  // codewords whose iteration l-1 satisfied every check stop there
-            int s = timed_launch(d, kClsSyn, st, "k_lane_update", [&] {
-                k_lane_update<W><<<lane_blocks, 128, 0, st>>>(d->done, ca.fail_prev, d->iters, d->conv, batch,
-                                                               l - 1, cap_iters, 1);
-            });
-            if (s != MLD_OK) return s;
-        }
-        va.want_bits = (last || (et && !fused)) ? 1 : 0;
+        va.want_bits = (last || et) ? 1 : 0;
         if (acc_mode) {
             // the check pass has formed L_v; the last iteration's decisions
             if (last && h.n_core > 0) {
@@ -351,7 +342,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
             });
             if (s != MLD_OK) return s;
         }
-        if ((et && !fused) || last) {
+        if (et || last) {
             int s = syndrome_round(l, et);
             if (s != MLD_OK) return s;
         }
@@ -366,6 +357,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
         });
         if (s != MLD_OK) return s;
     }
+    if (small && out_dev) return MLD_OK;
     const cudaMemcpyKind kind = out_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     MLD_CUDA(cudaMemcpyAsync(conv_out, d->conv, batch, kind, st));
     MLD_CUDA(cudaMemcpyAsync(iters_out, d->iters, sizeof(int32_t) * batch, kind, st));

@@ -55,12 +55,6 @@ void build_class_tables(mld_graph *g) {
             out.push_back(l);
         }
     }
-    // the fused syndrome check needs every check in a register class (the
-    // checks without edges and the irregular class are not covered)
-    g->fusable = true;
-    for (const mld::CheckClass &cl : g->h.classes)
-        if (cl.dc < 0 || cl.dd > 1 || cl.dc + cl.dd > mld::kMaxRegDeg || (cl.dc == 0 && cl.dd == 0))
-            g->fusable = false;
     // posterior accumulation: every check with edges in a register class
     g->acc_ok = true;
     for (const mld::CheckClass &cl : g->h.classes)
@@ -97,6 +91,7 @@ void decoder_free(mld_decoder *d) {
     if (d->cap) cudaStreamDestroy(d->cap);
     d->cap = nullptr;
     dfree(d->lctr);
+    dfree(d->bar);
 }
 
 // The device address of a page-locked, mapped host buffer; null for any
@@ -458,6 +453,7 @@ int mld_decoder_create(const mld_graph *g, const mld_opts *opts, mld_decoder **o
     if (s == MLD_OK) s = dalloc(&d->syn_stage, static_cast<size_t>(d->max_batch) * h.n_cn);
     if (s == MLD_OK) s = dalloc(&d->bits_stage, nb);
     if (s == MLD_OK) s = dalloc(&d->lctr, 2);
+    if (s == MLD_OK) s = dalloc(&d->bar, 3);
     if (s == MLD_OK) {
         cudaError_t ce = cudaStreamCreateWithFlags(&d->cap, cudaStreamNonBlocking);
         if (ce != cudaSuccess) s = cuda_fail(ce, "decoder_create: capture stream");
@@ -470,6 +466,7 @@ int mld_decoder_create(const mld_graph *g, const mld_opts *opts, mld_decoder **o
     }
     if (s == MLD_OK) {
         cudaError_t e2 = cudaMemset(d->status, 0, 4 * sizeof(int32_t));
+        if (e2 == cudaSuccess) e2 = cudaMemset(d->bar, 0, 3 * sizeof(uint32_t));
         if (e2 != cudaSuccess) s = cuda_fail(e2, "cudaMemset");
     }
     if (s != MLD_OK) {
@@ -707,6 +704,10 @@ extern "C" int mld_decode_noalloc(const mld_graph *g, int32_t msg_dtype, const f
     d.conv = base + L.conv;
     const bool et = (flags & MLD_EARLY_TERM) != 0;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    // the one-launch decode keeps its lane state on chip: its barrier takes the
+    // (256-byte aligned) place of the done words
+    d.bar = d.done;
+    MLD_CUDA(cudaMemsetAsync(d.bar, 0, 3 * sizeof(uint32_t), st));
     return msg_dtype == MLD_MSG_F16
                ? mld::run_decode_f16(&d, llr, nullptr, syndrome, batch, max_iters, et, bits_out, post_out,
                                     converged, iters_used, st, true)

@@ -342,14 +342,6 @@ struct CnArgs {
     const uint32_t *done;  // [slab][ceil(W/32)] converged lanes (ET)
     float lmax, amin;
     int final_pass, et;
-    // Fused syndrome check (early termination without soft output): this
-    // pass also forms the syndrome of the previous iteration from the signs
-    // of the posteriors it reads and the previous degree-1 decisions, and ORs
-    // the failing codewords into fail_prev.
-    int fuse;
-    int32_t batch;              // codewords (later lanes are padding)
-    const uint8_t *hb1_prev;    // degree-1 decisions of the previous iteration
-    uint32_t *fail_prev;        // [slab][ceil(W/32)] fail words of the previous iteration
     // Posterior accumulation (fixed iterations only): each new message, as
     // stored, is added to this [slab][n_core][W] array, which holds L_ch on
     // entry and L_v of this iteration (Eq. 4) once the pass is complete.
@@ -518,14 +510,11 @@ struct TermsRing {
 // .. lane0+3 of the slab; rout: its first message row there, e0 and s0 its
 // first core edge and degree-1 slot; valid false: compute but store nothing.  sb: the
 // check's syndrome bits for the 4 codewords (bit k: lane0 + k); donenib:
-// their converged flags under early termination.  FUSE (with kPassHard): with
-// a.fuse the call also returns the previous iteration's syndrome failures of
-// the check for the 4 codewords (bit k: codeword lane0 + k), else 0.  The
-// terms are read through t: lv(i) and ro(i), posterior and stored message of
+// their converged flags under early termination.  The terms are read through t: lv(i) and ro(i), posterior and stored message of
 // core term i, p1(i), phi term of degree-1 term i.  LAY (layered schedule):
 // the check also owns its core VNs' posteriors and updates them in place.
-template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC, bool FUSE, bool LAY, typename Terms>
-__device__ __forceinline__ uint32_t check_terms(const CnArgs &a, int lane0, int slab, bool valid, MsgT *rout,
+template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC, bool LAY, typename Terms>
+__device__ __forceinline__ void check_terms(const CnArgs &a, int lane0, int slab, bool valid, MsgT *rout,
                                                 int32_t e0, int32_t s0, uint32_t sb, uint32_t donenib, const Terms &t) {
     constexpr int NB = W / 8;
     constexpr int D = DC + DD;
@@ -540,7 +529,6 @@ __device__ __forceinline__ uint32_t check_terms(const CnArgs &a, int lane0, int 
     // q is its channel LLR, whose f was formed once on entry.
     float2 f[D][kP];
     uint32_t sg[D][kP], par[kP];
-    uint32_t lvs[kP] = {0u, 0u};  // sign parity of the posteriors read (fused syndrome)
 #pragma unroll
     for (int p = 0; p < kP; ++p) par[p] = sign_word_of_bits(sb >> (2 * p));
 #pragma unroll
@@ -548,10 +536,6 @@ __device__ __forceinline__ uint32_t check_terms(const CnArgs &a, int lane0, int 
         if (i < dc) {
             const float4 lv = t.lv(i);
             const float2 lp[kP] = {make_float2(lv.x, lv.y), make_float2(lv.z, lv.w)};
-            if constexpr (HARD1 && FUSE) {
-#pragma unroll
-                for (int p = 0; p < kP; ++p) lvs[p] ^= sign_word(lp[p]);
-            }
             const typename Msg<MsgT>::Raw ro = t.ro(i);
             // phi(|q|) floored at amin = phi(lmax) is phi of |q| clamped above at
             // lmax.  |q| is not clamped below: an argument under phi(lmax)
@@ -674,42 +658,6 @@ __device__ __forceinline__ uint32_t check_terms(const CnArgs &a, int lane0, int 
             for (int p = 0; p < kP; ++p) suf[p] = (i == D - 1) ? f[i][p] : add2(suf[p], f[i][p]);
         }
     }
-    uint32_t fail = 0;
-    if constexpr (HARD1 && FUSE) {
-        if (a.fuse && valid) {
-            // previous iteration: s_c XOR the decisions of the check's VNs
-            // (core: posterior < 0, the sign read above; degree-1: stored bit)
-            uint32_t x = sb & 0xFu;
-#pragma unroll
-            for (int kk = 0; kk < kK; ++kk) x ^= (sign_of(lvs[kk / 2], kk & 1) >> 31) << kk;
-            if (DD == 1)
-                x ^= (static_cast<uint32_t>(a.hb1_prev[(static_cast<size_t>(slab) * a.n_deg1 + s0) * NB + lane0 / 8]) >>
-                      (lane0 & 7)) & 0xFu;
-            const int lanes = a.batch - slab * W - lane0;  // real codewords among the 4
-            const uint32_t real = lanes >= kK ? 0xFu : (lanes > 0 ? (1u << lanes) - 1u : 0u);
-            fail = x & real & ~donenib;
-        }
-    }
-    return fail;
-}
-
-// ORs the fused syndrome failures of a block's threads (4 codewords each,
-// at lane0) into the fail words of the slab: warp reduction, then one atomic
-// per word and warp.  Every thread of the block must call it.
-template <int W>
-__device__ __forceinline__ void flush_fail(uint32_t *fail_slab, uint32_t nib, int lane0) {
-    constexpr int DW = (W + 31) / 32;
-    uint32_t lo = lane0 < 32 ? nib << lane0 : 0u;
-    uint32_t hi = lane0 >= 32 ? nib << (lane0 - 32) : 0u;
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        lo |= __shfl_xor_sync(0xFFFFFFFFu, lo, o);
-        if (DW > 1) hi |= __shfl_xor_sync(0xFFFFFFFFu, hi, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (lo) atomicOr(fail_slab, lo);
-        if (DW > 1 && hi) atomicOr(fail_slab + 1, hi);
-    }
 }
 
 // Checks of any degree, edges read through cptr/dptr; leave-one-out sums as
@@ -803,11 +751,10 @@ void allow_smem(K kernel) {
 // The threads of a class launch (t0: thread index in the slab's grid of
 // `blocks` blocks; smem: RingShape::kBytes bytes), each taking every
 // stride-th check with the same codewords; both threads of a shuffle pair
-// belong to one check and leave together.  With FUSE the fused syndrome
-// failures are ORed into a.fail_prev.  LAY: the launch's k-th check is
+// belong to one check and leave together.  LAY: the launch's k-th check is
 // pos[k], its messages start at layered edge cl.e0 + k DC (contiguous in the
 // launch), its degree-1 slots follow the class order.
-template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC = false, bool FUSE = false, bool LAY = false>
+template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC = false, bool LAY = false>
 __device__ __forceinline__ void check_class_body(const CnArgs &a, const ClassLaunch &cl, int64_t t0,
                                                  int32_t blocks, int slab, unsigned char *smem,
                                                  const int32_t *pos = nullptr) {
@@ -840,7 +787,6 @@ __device__ __forceinline__ void check_class_body(const CnArgs &a, const ClassLau
         cp_async_commit();  // (an empty group past the end keeps the count)
         sbn = sbp[static_cast<size_t>(LAY ? cn : min(j, cl.count - 1)) * NB];
     };
-    uint32_t fail = 0;
     int32_t j = static_cast<int32_t>(t0 / TPC);
     cols(j);
     request(j, 0);
@@ -854,23 +800,20 @@ __device__ __forceinline__ void check_class_body(const CnArgs &a, const ClassLau
         cols(j + 2 * stride);
         cp_async_wait<1>();
         const Ring t{smem + slot * kStage};
-        fail |= check_terms<MsgT, W, DC, DD, PASS, ACC, FUSE, LAY>(
+        check_terms<MsgT, W, DC, DD, PASS, ACC, LAY>(
             a, lane0, slab, true, rb + static_cast<size_t>(j * DC) * W, cl.e0 + j * DC, s0, sb, donenib, t);
-    }
-    if constexpr (FUSE) {
-        if (a.fuse) flush_fail<W>(a.fail_prev + slab * ((W + 31) / 32), fail, lane0);
     }
 }
 
 // One check class per launch, its shape (DC, DD) a compile-time constant: the
 // register arrays are sized exactly and only this class's code is hot.
-template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC = false, bool FUSE = false>
+template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC = false>
 __global__ void __launch_bounds__(kBlock, (kCheckBlocksPerSm<DC + DD>))
     k_check_update(CnArgs a, ClassLaunch cl) {
     const int slab = blockIdx.y;
     if (PASS != kPassPlain && a.et && slab_all_done<W>(a.done, slab)) return;  // block-uniform
     extern __shared__ __align__(128) unsigned char smem[];
-    check_class_body<MsgT, W, DC, DD, PASS, ACC, FUSE>(a, cl,
+    check_class_body<MsgT, W, DC, DD, PASS, ACC>(a, cl,
                                                   static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x,
                                                   static_cast<int32_t>(gridDim.x), slab, smem);
 }
@@ -979,7 +922,7 @@ struct TermsShared {
 };
 
 // A capped grid; block b takes stages b, b + gridDim.x, ...  Sum-product,
-// no fused syndrome (HARD1 false), no accumulation.  LSU false: each
+// not the decisions-only pass, no accumulation.  LSU false: each
 // posterior row is one bulk copy, issued by the thread that loaded its
 // column index; LSU true: every thread copies its own 16 bytes of each of
 // its check's posterior rows with cp.async (the load/store unit, not the
@@ -1096,7 +1039,7 @@ __global__ void __launch_bounds__(kBlock, kStagedBlocksPerSm) k_check_staged(CnA
         t.phi = reinterpret_cast<const float *>(base + S::kMsg) + g * DD * W + lane0;
         t.post = reinterpret_cast<const float *>(base + S::kMsg + S::kP1) + g * DC * W + lane0;
         MsgT *rout = static_cast<MsgT *>(a.r) + (static_cast<size_t>(slab) * a.e_core + cl.e0 + j * DC) * W + lane0;
-        check_terms<MsgT, W, DC, DD, kPassFull, false, false, false>(a, lane0, slab, valid, rout, cl.e0 + j * DC,
+        check_terms<MsgT, W, DC, DD, kPassFull, false, false>(a, lane0, slab, valid, rout, cl.e0 + j * DC,
                                                               cl.s0 + j * DD, sb, donenib, t);
         if (__syncthreads_or(!ok)) {
             // a copy never completed: record it, give the copies in flight
@@ -1130,8 +1073,8 @@ __global__ void __launch_bounds__(kBlock) k_check_update_irregular(CnArgs a, Cla
 // Classes with at most one degree-1 VN per check and at most kMaxRegDeg terms
 // run the register kernel for their shape; any other class (possible in
 // caller graphs, not in the MET ensembles) runs the streaming kernel.
-// hard1: early termination without soft output (degree-1 decisions only, and
-// the fused syndrome check when ca.fuse; see check_terms).  With ca.acc set
+// hard1: early termination without soft output (degree-1 decisions only).  With
+// ca.acc set
 // (fixed iterations, default slab width, register classes only) the kernels
 // also add every new message to the next posteriors.
 template <typename MsgT, int W>
@@ -1174,7 +1117,7 @@ void launch_staged(const CnArgs &ca, const ClassLaunch &cl, int slabs, cudaStrea
 }
 
 // The staged kernel, where it applies (half messages at slab width 64,
-// sum-product, no fused syndrome, no accumulation, a register class of at
+// sum-product, no accumulation, a register class of at
 // most six terms with at most one degree-1 VN per check); false otherwise.
 template <typename MsgT, int W>
 bool try_launch_staged(const CnArgs &ca, const ClassLaunch &cl, int slabs, cudaStream_t st, int staged_cap,
@@ -1225,8 +1168,7 @@ void launch_check_class(const CnArgs &ca, const ClassLaunch &cl, int slabs, cuda
                 return;                                                                             \
             }                                                                                       \
         }                                                                                           \
-        if (hard1 && ca.fuse) MLD_LAUNCH(DCV, DDV, kPassHard, false, true);                         \
-        else if (hard1) MLD_LAUNCH(DCV, DDV, kPassHard);                                            \
+        if (hard1) MLD_LAUNCH(DCV, DDV, kPassHard);                                            \
         else if (plain) MLD_LAUNCH(DCV, DDV, kPassPlain);                                           \
         else MLD_LAUNCH(DCV, DDV, kPassFull);                                                       \
         return;
@@ -1288,7 +1230,7 @@ __global__ void __launch_bounds__(kBlock, (kCheckBlocksPerSm<DC + DD>))
     const int slab = blockIdx.y;
     if (PASS != kPassPlain && a.et && slab_all_done<W>(a.done, slab)) return;  // block-uniform
     extern __shared__ __align__(128) unsigned char smem[];
-    check_class_body<MsgT, W, DC, DD, PASS, false, false, true>(
+    check_class_body<MsgT, W, DC, DD, PASS, false, true>(
         a, cl, static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x, static_cast<int32_t>(gridDim.x), slab, smem,
         pos);
 }
@@ -1716,8 +1658,7 @@ __device__ __forceinline__ void var_body(const VnArgs &a, int64_t t, int slab) {
     float4 o0 = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y), o1 = make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y);
     float *lv = a.Lv + vrow;
     if (a.et) {
-        // converged lanes keep the posterior of their last iteration (with a
-        // fused syndrome check a lane is marked after its messages moved on)
+        // converged lanes keep the posterior of their last iteration
         constexpr int DW = (W + 31) / 32;
         const uint32_t dn = (a.done[slab * DW + lane0 / 32] >> (lane0 & 31)) & 0xFFu;
         if (dn) {
@@ -2047,11 +1988,6 @@ __device__ __forceinline__ void interleave_body(const InArgs &a, int tile_x, int
     }
 }
 
-template <int W, int F>
-__global__ void __launch_bounds__(kBlock) k_interleave_in(InArgs a) {
-    interleave_body<W, F>(a, blockIdx.x, blockIdx.y);
-}
-
 template <int W>
 __device__ __forceinline__ void syndrome_in_body(const uint8_t *syn, const int32_t *cint, int32_t n_cn,
                                                  int32_t batch, uint8_t *sbits, int tile_x, int slab) {
@@ -2076,10 +2012,28 @@ __device__ __forceinline__ void syndrome_in_body(const uint8_t *syn, const int32
     }
 }
 
-template <int W>
-__global__ void __launch_bounds__(kBlock) k_syndrome_in(const uint8_t *syn, const int32_t *cint, int32_t n_cn,
-                                                        int32_t batch, uint8_t *sbits) {
-    syndrome_in_body<W>(syn, cint, n_cn, batch, sbits, blockIdx.x, blockIdx.y);
+// Everything a decode needs before its first iteration, in one launch: the
+// blocks x < in_tiles transpose 32 VNs x W codewords of slab y, the others 32
+// checks' syndrome bits, and all of them clear their share of the messages.
+struct PrologueArgs {
+    InArgs in;
+    const uint8_t *syn;
+    const int32_t *cint;
+    uint8_t *sbits;
+    int32_t n_cn, in_tiles;
+    uint4 *r;    // messages of all slabs
+    size_t r16;  // their size in 16-byte words
+};
+
+template <int W, int F>
+__global__ void __launch_bounds__(kBlock) k_prologue(PrologueArgs a) {
+    const size_t blocks = static_cast<size_t>(gridDim.x) * gridDim.y;
+    const size_t share = (a.r16 + blocks - 1) / blocks;
+    const size_t r0 = (static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * share;
+    for (size_t i = r0 + threadIdx.x; i < min(r0 + share, a.r16); i += blockDim.x) a.r[i] = make_uint4(0, 0, 0, 0);
+    const int x = blockIdx.x;
+    if (x < a.in_tiles) interleave_body<W, F>(a.in, x, blockIdx.y);
+    else syndrome_in_body<W>(a.syn, a.cint, a.n_cn, a.in.batch, a.sbits, x - a.in_tiles, blockIdx.y);
 }
 
 // bit-sliced hard decisions of a float array [slab][count][W] -> [slab][count][W/8]
@@ -2260,6 +2214,7 @@ struct mld_decoder {
     // variant and layering of the graph)
     cudaStream_t cap = nullptr;
     int32_t *lctr = nullptr;
+    uint32_t *bar = nullptr;  // grid barrier of the one-launch decode (3 words, zero between launches)
     struct LoopGraph { int32_t batch, variant; uint64_t layers_gen; cudaGraphExec_t exec; };
     std::vector<LoopGraph> loops;
     float *Lv2 = nullptr, *Lv3 = nullptr;
@@ -2289,6 +2244,13 @@ int run_decode_f16(mld_decoder *d, const float *in, const float *sigma, const ui
 int run_decode_f32(mld_decoder *d, const float *in, const float *sigma, const uint8_t *syn, int32_t batch,
                    int32_t iters, bool et, uint8_t *bits, float *post, uint8_t *conv, int32_t *it,
                    cudaStream_t st, bool out_dev);
+// small_f16.cu / small_f32.cu: the iterations of a small flooding sum-product
+// decode in one cooperative launch; false if it does not apply (nothing was
+// enqueued).  iters_out / conv_out: the caller's device arrays or null.
+bool small_decode_f16(mld_decoder *d, int W, int32_t batch, int32_t iters, bool et, bool hard1, int32_t *iters_out,
+                      uint8_t *conv_out, int sm_count, cudaStream_t st);
+bool small_decode_f32(mld_decoder *d, int W, int32_t batch, int32_t iters, bool et, bool hard1, int32_t *iters_out,
+                      uint8_t *conv_out, int sm_count, cudaStream_t st);
 // Sets the shared-memory carveout of the staged kernels that decode_f16.cu
 // launches (a function attribute belongs to one translation unit's kernel).
 cudaError_t prepare_staged_f16();

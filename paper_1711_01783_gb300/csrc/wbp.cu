@@ -535,17 +535,14 @@ int wbp_forward_w(mld_decoder *d, const float *llr, const uint8_t *syn, int32_t 
     const mld::HostGraph &h = d->g->h;
     const int slabs = (batch + W - 1) / W;
     const size_t rsz = static_cast<size_t>(slabs) * h.e_core * W;
-    if (rsz) MLD_CUDA(cudaMemsetAsync(d->r, 0, rsz * sizeof(float), st));
     // weighted BP works in nats: no scaling on entry or exit
     InArgs ia{llr, nullptr, d->g->unit, h.n_vn, h.n_core, h.n_deg1, batch, d->lmax, 1.f, d->lmax, d->amin,
               d->lch, d->Lv, d->lch1, d->post1, d->phi1};
-    if (h.n_vn > 0) {
-        k_interleave_in<W, kFitNat><<<dim3((h.n_vn + 31) / 32, slabs), kBlock, 0, st>>>(ia);
-        MLD_LAUNCHED("k_interleave_in");
-    }
-    if (h.n_cn > 0) {
-        k_syndrome_in<W><<<dim3((h.n_cn + 31) / 32, slabs), kBlock, 0, st>>>(syn, d->g->cint, h.n_cn, batch, d->sbits);
-        MLD_LAUNCHED("k_syndrome_in");
+    const PrologueArgs pa{ia, syn, d->g->cint, d->sbits, h.n_cn, (h.n_vn + 31) / 32, static_cast<uint4 *>(d->r),
+                          rsz * sizeof(float) / 16};
+    if (h.n_vn > 0 || h.n_cn > 0) {
+        k_prologue<W, kFitNat><<<dim3(pa.in_tiles + (h.n_cn + 31) / 32, slabs), kBlock, 0, st>>>(pa);
+        MLD_LAUNCHED("k_prologue");
     }
     const WArgs wa = wargs(d, w, n_types);
     auto iters = [&](cudaStream_t s2) {
