@@ -516,7 +516,6 @@ struct TermsRing {
 template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC, bool LAY, typename Terms>
 __device__ __forceinline__ void check_terms(const CnArgs &a, int lane0, int slab, bool valid, MsgT *rout,
                                                 int32_t e0, int32_t s0, uint32_t sb, uint32_t donenib, const Terms &t) {
-    constexpr int NB = W / 8;
     constexpr int D = DC + DD;
     constexpr int dc = DC;
     constexpr bool HARD1 = PASS == kPassHard;

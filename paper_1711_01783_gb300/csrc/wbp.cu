@@ -27,7 +27,325 @@ struct WArgs {
     float lmax, amin;
 };
 
-__device__ __forceinline__ float inv_sinh(float x) { return 1.0f / sinhf(x); }
+// 1 / sinh x for 0 < x: below 0.5 the reciprocal of sinh's Taylor polynomial
+// (remainder x^8 / 9!, 1e-8 relative), above 2 e / (1 - e^2) with e = exp(-x),
+// formed as 2^-(x log2 e) with the product's rounding error put back.  One
+// reciprocal and no branch: sinhf and a division took most of the adjoint's
+// instructions.
+__device__ __forceinline__ float inv_sinh(float x) {
+    const float y = x * 1.44269502f;
+    const float lo = fmaf(x, 1.92596303e-8f, fmaf(x, 1.44269502f, -y));
+    const float e = mufu_ex2(-y) * fmaf(lo, -0.693147181f, 1.f);
+    const float t = x * x;
+    const float poly = fmaf(t, fmaf(t, fmaf(t, 1.f / 5040.f, 1.f / 120.f), 1.f / 6.f), 1.f);
+    const bool near = x < 0.5f;
+    const float den = near ? x * poly : fmaf(-e, e, 1.f);
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(den));
+    return near ? r : (e + e) * r;
+}
+
+// phi of two values in nats: phi_f<kFitNat> on packed pairs, same roundings.
+__device__ __forceinline__ float2 phi2_nat(float2 x) {
+    auto both = [](float v) { return make_float2(v, v); };
+    const float kLn2 = 0.693147180559945309f;
+    const float2 t = __fmul2_rn(x, x);
+    float2 ps = __ffma2_rn(both(-MLD_PHI_S4), t, both(-MLD_PHI_S3));
+    ps = __ffma2_rn(ps, t, both(-MLD_PHI_S2));
+    ps = __ffma2_rn(ps, t, both(-MLD_PHI_S1));
+    ps = __ffma2_rn(ps, t, both(-MLD_PHI_S0));
+    const float2 lg = make_float2(mufu_lg2(x.x), mufu_lg2(x.y));
+    const float2 small = __ffma2_rn(t, ps, __ffma2_rn(both(-kLn2), lg, both(kLn2)));
+    const float2 y = __fmul2_rn(x, both(-1.442695040888963407f));
+    const float2 e = make_float2(mufu_ex2(y.x), mufu_ex2(y.y));
+    const float2 z = __fmul2_rn(e, e);
+    float2 pl = __ffma2_rn(both(MLD_PHI_L3), z, both(MLD_PHI_L2));
+    pl = __ffma2_rn(pl, z, both(MLD_PHI_L1));
+    pl = __ffma2_rn(pl, z, both(MLD_PHI_L0));
+    const float2 large = __fmul2_rn(e, pl);
+    return make_float2(sel_lt(x.x, MLD_PHI_X0, small.x, large.x), sel_lt(x.y, MLD_PHI_X0, small.y, large.y));
+}
+
+__device__ __forceinline__ float2 clamp2(float2 x, float lo, float hi) {
+    return make_float2(clampf(x.x, lo, hi), clampf(x.y, lo, hi));
+}
+__device__ __forceinline__ float2 pair_of(const float4 &v, int p) {
+    return p == 0 ? make_float2(v.x, v.y) : make_float2(v.z, v.w);
+}
+
+// ---------------------------------------------------------------------------
+// Check kernels of the register classes: one launch covers every class of the
+// graph, a block finds its class in a table and runs the body of its shape
+// (DC core edges, DD degree-1 VNs), with every operand of a check requested
+// before any arithmetic and the arithmetic two codewords at a time.
+// ---------------------------------------------------------------------------
+constexpr int kMaxTable = 16;
+struct ClassTable {
+    mld::ClassLaunch cls[kMaxTable];
+    int32_t first[kMaxTable + 1];  // first block of each class, and the end
+    int n;
+};
+
+// Operands of one check for 4 codewords.
+template <int W, int DC, int DD>
+struct CheckOps {
+    static constexpr int D = DC + DD;
+    float4 lv[DC > 0 ? DC : 1], ro[DC > 0 ? DC : 1], l1[DD > 0 ? DD : 1];
+    float wt[D];
+    int ty[D];
+    uint32_t sb;
+
+    // rp: the messages of the previous iteration, null for none (all zero)
+    __device__ __forceinline__ void load(const WArgs &a, const mld::ClassLaunch &cl, int32_t j, int slab, int lane0,
+                                         int t, const float *rp, const float *lvp) {
+        constexpr int NB = W / 8;
+        const int32_t c = cl.c0 + j, e0 = cl.e0 + j * DC, s0 = cl.s0 + j * DD;
+#pragma unroll
+        for (int i = 0; i < DC; ++i) {
+            lv[i] = ldf4(lvp + (static_cast<size_t>(slab) * a.n_core + __ldg(a.col + e0 + i)) * W + lane0);
+            ro[i] = rp ? *reinterpret_cast<const float4 *>(rp + (static_cast<size_t>(slab) * a.e_core + e0 + i) * W + lane0)
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
+            ty[i] = a.et_core[e0 + i];
+        }
+#pragma unroll
+        for (int i = 0; i < DD; ++i) {
+            l1[i] = ldf4(a.lch1 + (static_cast<size_t>(slab) * a.n_deg1 + s0 + i) * W + lane0);
+            ty[DC + i] = a.et_deg1[s0 + i];
+        }
+        sb = static_cast<uint32_t>(a.sbits[(static_cast<size_t>(slab) * a.n_cn + c) * NB + lane0 / 8]) >> (lane0 & 7);
+        const float *row = a.w + static_cast<size_t>(t - 1) * a.n_types;
+#pragma unroll
+        for (int i = 0; i < D; ++i) wt[i] = __ldg(row + ty[i]);
+    }
+    // x_e of pair p: posterior minus own message (degree-1 VN: channel LLR)
+    __device__ __forceinline__ float2 x(int i, int p) const {
+        return i < DC ? sub2(pair_of(lv[i], p), pair_of(ro[i], p)) : pair_of(l1[i - DC], p);
+    }
+};
+
+// The forward quantities of one pair of codewords.
+template <int D>
+struct PairState {
+    float2 q[D], f[D], pre[D];
+    float2 sg;  // product of signs and syndrome sign over all terms
+    template <typename Ops>
+    __device__ __forceinline__ void forward(const Ops &ops, const WArgs &a, int p) {
+        sg = make_float2((ops.sb >> (2 * p)) & 1u ? -1.f : 1.f, (ops.sb >> (2 * p + 1)) & 1u ? -1.f : 1.f);
+        float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            q[i] = clamp2(__fmul2_rn(make_float2(ops.wt[i], ops.wt[i]), ops.x(i, p)), -a.lmax, a.lmax);
+            f[i] = phi2_nat(clamp2(make_float2(fabsf(q[i].x), fabsf(q[i].y)), a.amin, a.lmax));
+            if (q[i].x < 0.f) sg.x = -sg.x;
+            if (q[i].y < 0.f) sg.y = -sg.y;
+            pre[i] = acc;
+            acc = add2(acc, f[i]);
+        }
+    }
+    // sign of the other terms' product
+    __device__ __forceinline__ float2 others(int i) const {
+        return make_float2(q[i].x < 0.f ? -sg.x : sg.x, q[i].y < 0.f ? -sg.y : sg.y);
+    }
+};
+
+// Forward check update of iteration t, codewords lane0 .. lane0+3: messages
+// r_in (null: zero) and posteriors lv of iteration t-1 to messages r_out (which
+// may be r_in); degree-1 posteriors written when `last`.
+template <int W, int DC, int DD>
+__device__ __forceinline__ void wbp_fwd(const WArgs &a, const mld::ClassLaunch &cl, int32_t j, int slab, int lane0,
+                                        const float *r_in, float *r_out, const float *lv, float *post1, int t, int last) {
+    constexpr int D = DC + DD;
+    CheckOps<W, DC, DD> ops;
+    ops.load(a, cl, j, slab, lane0, t, r_in, lv);
+    float2 out[D][kP];
+#pragma unroll
+    for (int p = 0; p < kP; ++p) {
+        PairState<D> s;
+        s.forward(ops, a, p);
+        float2 suf = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = D - 1; i >= 0; --i) {
+            if (i < DC || last) {
+                const float2 m = phi2_nat(clamp2(add2(s.pre[i], suf), a.amin, a.lmax));
+                out[i][p] = __fmul2_rn(s.others(i), make_float2(fminf(m.x, a.lmax), fminf(m.y, a.lmax)));
+            }
+            suf = add2(suf, s.f[i]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < DC; ++i)
+        *reinterpret_cast<float4 *>(r_out + (static_cast<size_t>(slab) * a.e_core + cl.e0 + j * DC + i) * W + lane0) =
+            make_float4(out[i][0].x, out[i][0].y, out[i][1].x, out[i][1].y);
+    if (last) {
+#pragma unroll
+        for (int i = 0; i < DD; ++i) {
+            const float4 l = ops.l1[i];
+            *reinterpret_cast<float4 *>(post1 + (static_cast<size_t>(slab) * a.n_deg1 + cl.s0 + j * DD + i) * W + lane0) =
+                make_float4(l.x + out[DC + i][0].x, l.y + out[DC + i][0].y, l.z + out[DC + i][1].x,
+                            l.w + out[DC + i][1].y);
+        }
+    }
+}
+
+// Adjoint of the check update of iteration t for 4 codewords.  dloss/dr^t of
+// core edge e is G_v(e) - gx_e with gx the dloss/dx^{t+1} that this pass then
+// replaces by dloss/dx^t (G, gx_used: see the launches); gd1: of the degree-1
+// edges (only at t = T; else null).  glch1 accumulates dloss/dL_ch of the
+// degree-1 VNs, gw the weight gradients per edge type.
+template <int W, int DC, int DD>
+__device__ __forceinline__ void wbp_bwd(const WArgs &a, const mld::ClassLaunch &cl, int32_t j, int slab, int lane0,
+                                        const float *rp, const float *lvp, const float *G, bool gx_used, float *gx,
+                                        const float *gd1, float *glch1, int t, float (&gw)[kMaxTypes]) {
+    constexpr int D = DC + DD;
+    const int32_t e0 = cl.e0 + j * DC, s0 = cl.s0 + j * DD;
+    CheckOps<W, DC, DD> ops;
+    ops.load(a, cl, j, slab, lane0, t, rp, lvp);
+    float *gxr = gx + (static_cast<size_t>(slab) * a.e_core + e0) * W + lane0;
+    const size_t d0 = (static_cast<size_t>(slab) * a.n_deg1 + s0) * W + lane0;
+    float4 g[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        if (i < DC) {
+            g[i] = ldf4(G + (static_cast<size_t>(slab) * a.n_core + __ldg(a.col + e0 + i)) * W + lane0);
+            if (gx_used) {
+                const float4 o = *reinterpret_cast<const float4 *>(gxr + i * W);
+                g[i] = make_float4(g[i].x - o.x, g[i].y - o.y, g[i].z - o.z, g[i].w - o.w);
+            }
+        } else {
+            g[i] = gd1 ? ldf4(gd1 + d0 + (i - DC) * W) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    float gwi[D];
+    float2 out[D][kP];
+#pragma unroll
+    for (int i = 0; i < D; ++i) gwi[i] = 0.f;
+#pragma unroll
+    for (int p = 0; p < kP; ++p) {
+        PairState<D> s;
+        s.forward(ops, a, p);
+        // g_o_i = sign_i * g_r_i * phi'(o_i) where o_i is strictly inside the clamp
+        float2 go[D], suf = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = D - 1; i >= 0; --i) {
+            const float2 o = add2(s.pre[i], suf), sgn = s.others(i), gi = pair_of(g[i], p);
+            go[i].x = (o.x > a.amin && o.x < a.lmax) ? -sgn.x * gi.x * inv_sinh(o.x) : 0.f;
+            go[i].y = (o.y > a.amin && o.y < a.lmax) ? -sgn.y * gi.y * inv_sinh(o.y) : 0.f;
+            suf = add2(suf, s.f[i]);
+        }
+        // g_f_j = sum_{i != j} g_o_i (prefix + suffix), then back through phi,
+        // |.|, the clamps (outside them |q| is amin or below, or lmax) and the weight
+        float2 gpre[D], acc = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            gpre[i] = acc;
+            acc = add2(acc, go[i]);
+        }
+        float2 gsuf = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = D - 1; i >= 0; --i) {
+            const float2 gf = add2(gpre[i], gsuf), x = ops.x(i, p);
+            gsuf = add2(gsuf, go[i]);
+            auto through = [&](float q, float gfk) {
+                const float aq = fabsf(q);
+                const float ga = (aq > a.amin && aq < a.lmax) ? -gfk * inv_sinh(aq) : 0.f;
+                return q < 0.f ? -ga : ga;
+            };
+            const float2 gp = make_float2(through(s.q[i].x, gf.x), through(s.q[i].y, gf.y));
+            gwi[i] = fmaf(gp.y, x.y, fmaf(gp.x, x.x, gwi[i]));
+            out[i][p] = make_float2(gp.x * ops.wt[i], gp.y * ops.wt[i]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+#pragma unroll
+        for (int k = 0; k < kMaxTypes; ++k) gw[k] += (k == ops.ty[i]) ? gwi[i] : 0.f;
+        const float4 v = make_float4(out[i][0].x, out[i][0].y, out[i][1].x, out[i][1].y);
+        if (i < DC) {
+            *reinterpret_cast<float4 *>(gxr + i * W) = v;
+        } else {
+            float4 *pp = reinterpret_cast<float4 *>(glch1 + d0 + (i - DC) * W);
+            float4 o = *pp;
+            o.x += v.x; o.y += v.y; o.z += v.z; o.w += v.w;
+            *pp = o;
+        }
+    }
+}
+
+// The block's class and its thread's check; false past the class's end.
+template <int W>
+__device__ __forceinline__ bool table_check(const ClassTable &tb, int &k, int32_t &j, int &lane0) {
+    constexpr int TPC = W / kK;
+    k = 0;
+    while (static_cast<int32_t>(blockIdx.x) >= tb.first[k + 1]) ++k;
+    const int32_t lt = (static_cast<int32_t>(blockIdx.x) - tb.first[k]) * kBlock + static_cast<int32_t>(threadIdx.x);
+    j = lt / TPC;
+    lane0 = (lt % TPC) * kK;
+    return j < tb.cls[k].count;
+}
+
+#define MLD_WBP_SHAPES(X)                                                              \
+    X(1, 0) X(2, 0) X(3, 0) X(4, 0) X(5, 0) X(6, 0) X(7, 0) X(8, 0)                     \
+    X(0, 1) X(1, 1) X(2, 1) X(3, 1) X(4, 1) X(5, 1) X(6, 1) X(7, 1)
+
+template <int W>
+__global__ void __launch_bounds__(kBlock, 4) kw_fwd(WArgs a, ClassTable tb, const float *r_in, float *r_out,
+                                                    const float *lv, float *post1, int t, int last) {
+    int k, lane0;
+    int32_t j;
+    if (!table_check<W>(tb, k, j, lane0)) return;
+    const mld::ClassLaunch &cl = tb.cls[k];
+    switch (cl.dc * 2 + (cl.deg - cl.dc)) {
+#define X(DC, DD) \
+    case (DC) * 2 + (DD): wbp_fwd<W, DC, DD>(a, cl, j, blockIdx.y, lane0, r_in, r_out, lv, post1, t, last); break;
+        MLD_WBP_SHAPES(X)
+#undef X
+        default: break;
+    }
+}
+
+// Block partial sums of the weight gradient (deterministic order) into row
+// `row` of gwp.  Every thread of the block must call it.
+__device__ __forceinline__ void block_weight_sums(const float (&gw)[kMaxTypes], int n_types, float *gwp, size_t row) {
+    __shared__ float red[kBlock / 32][kMaxTypes];
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+#pragma unroll
+    for (int k = 0; k < kMaxTypes; ++k) {
+        if (k < n_types) {
+            float v = gw[k];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+            if (lane == 0) red[warp][k] = v;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < n_types) {
+        float v = 0.f;
+        for (int i = 0; i < kBlock / 32; ++i) v += red[i][threadIdx.x];
+        gwp[row * n_types + threadIdx.x] = v;
+    }
+}
+
+template <int W>
+__global__ void __launch_bounds__(kBlock, 3) kw_bwd(WArgs a, ClassTable tb, const float *rp, const float *lvp,
+                                                    const float *G, int gx_used, float *gx, const float *gd1,
+                                                    float *glch1, float *gwp, int t) {
+    float gw[kMaxTypes];
+#pragma unroll
+    for (int k = 0; k < kMaxTypes; ++k) gw[k] = 0.f;
+    int k, lane0;
+    int32_t j;
+    if (table_check<W>(tb, k, j, lane0)) {
+        const mld::ClassLaunch &cl = tb.cls[k];
+        switch (cl.dc * 2 + (cl.deg - cl.dc)) {
+#define X(DC, DD)                                                                                                  \
+    case (DC) * 2 + (DD):                                                                                          \
+        wbp_bwd<W, DC, DD>(a, cl, j, blockIdx.y, lane0, rp, lvp, G, gx_used != 0, gx, gd1, glch1, t, gw); break;
+            MLD_WBP_SHAPES(X)
+#undef X
+            default: break;
+        }
+    }
+    block_weight_sums(gw, a.n_types, gwp, static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x);
+}
 
 // Recomputes the forward quantities of one check (at most DMAX terms) for 4
 // codewords at iteration t from r^{t-1} (rp) and L_v^{t-1} (lvp).  Loops run
@@ -62,7 +380,8 @@ struct CheckState {
             if (i < nce) {
                 const int32_t e = e0 + i;
                 const float4 lv = ldf4(lvp + (static_cast<size_t>(slab) * a.n_core + a.col[e]) * W + lane0);
-                const float4 ro = ldf4(rp + (static_cast<size_t>(slab) * a.e_core + e) * W + lane0);
+                const float4 ro = rp ? ldf4(rp + (static_cast<size_t>(slab) * a.e_core + e) * W + lane0)
+                                     : make_float4(0.f, 0.f, 0.f, 0.f);
                 xv = make_float4(lv.x - ro.x, lv.y - ro.y, lv.z - ro.z, lv.w - ro.w);
                 ty[i] = a.et_core[e];
             } else {
@@ -84,12 +403,10 @@ struct CheckState {
     }
 };
 
-// Forward check update of iteration t for checks c0 .. c0+count-1 of at most
-// DMAX terms (messages updated in place; degree-1 posteriors written when
-// `last`).  The loops run to the compile-time DMAX with the check's degree
-// as a guard, so the per-term arrays stay in registers for small DMAX.
+// Forward check update of checks of any degree up to DMAX (edges through
+// cptr / dptr), for the classes without a register shape.
 template <int W, int DMAX>
-__global__ void __launch_bounds__(kBlock) kw_check_fwd(WArgs a, float *r, const float *lv, float *post1, int t,
+__global__ void __launch_bounds__(kBlock) kw_check_fwd(WArgs a, const float *r_in, float *r, const float *lv, float *post1, int t,
                                                        int last, int32_t c0, int32_t count) {
     constexpr int TPC = W / kK;
     constexpr int NB = W / 8;
@@ -115,7 +432,9 @@ __global__ void __launch_bounds__(kBlock) kw_check_fwd(WArgs a, float *r, const 
             if (i < nce) {
                 const int32_t e = e0 + i;
                 const float4 l = ldf4(lv + (static_cast<size_t>(slab) * a.n_core + a.col[e]) * W + lane0);
-                const float4 ro = ldf4(r + (static_cast<size_t>(slab) * a.e_core + e) * W + lane0);
+                const float4 ro =
+                    r_in ? *reinterpret_cast<const float4 *>(r_in + (static_cast<size_t>(slab) * a.e_core + e) * W + lane0)
+                         : make_float4(0.f, 0.f, 0.f, 0.f);
                 xv = make_float4(l.x - ro.x, l.y - ro.y, l.z - ro.z, l.w - ro.w);
                 wt = wt_row[a.et_core[e]];
             } else {
@@ -160,33 +479,49 @@ __global__ void __launch_bounds__(kBlock) kw_check_fwd(WArgs a, float *r, const 
     }
 }
 
-// Forward check update of one class: DMAX = the class's degree (at most
-// kMaxRegDeg), or kMaxTerms for the irregular class.
-template <int W>
-void launch_check_fwd(const WArgs &wa, const mld::ClassLaunch &cl, float *r, const float *lv, float *post1, int t,
-                      int last, int slabs, cudaStream_t st) {
-    const dim3 grid(cl.blocks, slabs);
-    switch (cl.deg) {
-#define MLD_FWD(DV) \
-        case DV: kw_check_fwd<W, DV><<<grid, kBlock, 0, st>>>(wa, r, lv, post1, t, last, cl.c0, cl.count); return;
-        MLD_FWD(1) MLD_FWD(2) MLD_FWD(3) MLD_FWD(4) MLD_FWD(5) MLD_FWD(6) MLD_FWD(7) MLD_FWD(8)
-#undef MLD_FWD
-        default: kw_check_fwd<W, kMaxTerms><<<grid, kBlock, 0, st>>>(wa, r, lv, post1, t, last, cl.c0, cl.count);
+// Launches of one check pass: the register classes together, any other class
+// by itself.
+struct WbpClasses {
+    ClassTable table;
+    std::vector<mld::ClassLaunch> other;
+    int32_t parts = 0;  // blocks of an adjoint pass over one slab
+};
+
+WbpClasses wbp_classes(const std::vector<mld::ClassLaunch> &launches) {
+    WbpClasses c{};
+    for (const mld::ClassLaunch &cl : launches) {
+        const int dd = cl.deg - cl.dc;
+        const bool shaped = cl.dc >= 0 && (dd == 0 || dd == 1) && cl.deg <= mld::kMaxRegDeg;
+        if (shaped && c.table.n < kMaxTable) {
+            c.table.cls[c.table.n] = cl;
+            c.table.first[c.table.n + 1] = c.table.first[c.table.n] + cl.blocks;
+            c.table.n++;
+        } else {
+            c.other.push_back(cl);
+        }
+        c.parts += cl.blocks;
     }
+    return c;
 }
 
-// Adjoint of the check update of iteration t.
-//   gr   : dloss/dr^t for core edges (read)
-//   gd1  : dloss/dr^t of degree-1 edges (only at t = T; else null)
-//   gx   : dloss/dx^t for core edges (written)
-//   glch1: dloss/dL_ch of degree-1 VNs (accumulated)
-//   gwp  : per-block partial dloss/dw[t][type] (written, [gridDim.x*gridDim.y][n_types])
+template <int W>
+void launch_fwd(const WArgs &wa, const WbpClasses &c, const float *r_in, float *r_out, const float *lv, float *post1,
+                int t, int last, int slabs, cudaStream_t st) {
+    if (c.table.n)
+        kw_fwd<W><<<dim3(c.table.first[c.table.n], slabs), kBlock, 0, st>>>(wa, c.table, r_in, r_out, lv, post1, t, last);
+    for (const mld::ClassLaunch &cl : c.other)
+        kw_check_fwd<W, kMaxTerms><<<dim3(cl.blocks, slabs), kBlock, 0, st>>>(wa, r_in, r_out, lv, post1, t, last, cl.c0,
+                                                                            cl.count);
+}
+
+// Adjoint check update of checks of any degree up to DMAX (see wbp_bwd), for
+// the classes without a register shape; block partials from row part0 of gwp.
 template <int W, int DMAX>
-__global__ void __launch_bounds__(kBlock) kw_check_bwd(WArgs a, const float *rp, const float *lvp, const float *gr,
-                                                       const float *gd1, float *gx, float *glch1, float *gwp, int t,
+__global__ void __launch_bounds__(kBlock) kw_check_bwd(WArgs a, const float *rp, const float *lvp, const float *G,
+                                                       int gx_used, float *gx, const float *gd1, float *glch1,
+                                                       float *gwp, int t,
                                                        int32_t c0, int32_t count, int32_t part0) {
     constexpr int TPC = W / kK;
-    __shared__ float red[kBlock / 32][kMaxTypes];
     const int slab = blockIdx.y;
     const int64_t lt = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     float gw[kMaxTypes];
@@ -205,9 +540,14 @@ __global__ void __launch_bounds__(kBlock) kw_check_bwd(WArgs a, const float *rp,
             if (i >= s.deg) continue;
             const bool core = i < s.nce;
             float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (core)
-                g = ldf4(gr + (static_cast<size_t>(slab) * a.e_core + s.e0 + i) * W + lane0);
-            else if (gd1)
+            if (core) {
+                g = ldf4(G + (static_cast<size_t>(slab) * a.n_core + __ldg(a.col + s.e0 + i)) * W + lane0);
+                if (gx_used) {
+                    const float4 o = *reinterpret_cast<const float4 *>(
+                        gx + (static_cast<size_t>(slab) * a.e_core + s.e0 + i) * W + lane0);
+                    g = make_float4(g.x - o.x, g.y - o.y, g.z - o.z, g.w - o.w);
+                }
+            } else if (gd1)
                 g = ldf4(gd1 + (static_cast<size_t>(slab) * a.n_deg1 + s.s0 + i - s.nce) * W + lane0);
 #pragma unroll
             for (int k = 0; k < kK; ++k) {
@@ -260,90 +600,63 @@ __global__ void __launch_bounds__(kBlock) kw_check_bwd(WArgs a, const float *rp,
             }
         }
     }
-    // block partial sums of the weight gradient (deterministic order)
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    for (int k = 0; k < a.n_types; ++k) {
-        float v = gw[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-        if (lane == 0) red[warp][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < a.n_types) {
-        float v = 0.f;
-        for (int i = 0; i < kBlock / 32; ++i) v += red[i][threadIdx.x];
-        gwp[(static_cast<size_t>(part0) + static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x) * a.n_types +
-            threadIdx.x] = v;
-    }
+    block_weight_sums(gw, a.n_types, gwp,
+                      static_cast<size_t>(part0) + static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x);
 }
 
-// Adjoint check update of one class; its block partials start at part0.
 template <int W>
-void launch_check_bwd(const WArgs &wa, const mld::ClassLaunch &cl, const float *rp, const float *lvp,
-                      const float *gr, const float *gd1, float *gx, float *glch1, float *gwp, int t, int slabs,
-                      int32_t part0, cudaStream_t st) {
-    const dim3 grid(cl.blocks, slabs);
-    switch (cl.deg) {
-#define MLD_BWD(DV)                                                                                         \
-        case DV:                                                                                            \
-            kw_check_bwd<W, DV><<<grid, kBlock, 0, st>>>(wa, rp, lvp, gr, gd1, gx, glch1, gwp, t, cl.c0,    \
-                                                         cl.count, part0);                                  \
-            return;
-        MLD_BWD(1) MLD_BWD(2) MLD_BWD(3) MLD_BWD(4) MLD_BWD(5) MLD_BWD(6) MLD_BWD(7) MLD_BWD(8)
-#undef MLD_BWD
-        default:
-            kw_check_bwd<W, kMaxTerms><<<grid, kBlock, 0, st>>>(wa, rp, lvp, gr, gd1, gx, glch1, gwp, t, cl.c0,
-                                                                cl.count, part0);
+void launch_bwd(const WArgs &wa, const WbpClasses &c, const float *rp, const float *lvp, const float *G, int gx_used,
+                float *gx, const float *gd1, float *glch1, float *gwp, int t, int slabs, cudaStream_t st) {
+    int32_t part0 = 0;
+    if (c.table.n) {
+        const int32_t blocks = c.table.first[c.table.n];
+        kw_bwd<W><<<dim3(blocks, slabs), kBlock, 0, st>>>(wa, c.table, rp, lvp, G, gx_used, gx, gd1, glch1, gwp, t);
+        part0 = blocks * slabs;
+    }
+    for (const mld::ClassLaunch &cl : c.other) {
+        kw_check_bwd<W, kMaxTerms><<<dim3(cl.blocks, slabs), kBlock, 0, st>>>(wa, rp, lvp, G, gx_used, gx, gd1, glch1,
+                                                                            gwp, t, cl.c0, cl.count, part0);
+        part0 += cl.blocks * slabs;
     }
 }
 
 // Adjoint of x_e^t = L_ch(v) + sum_{e' != e} r_{e'}^{t-1} at core VN v:
-// G = sum_e gx_e; dL_ch += G; dr_{e'}^{t-1} = G - gx_{e'} (when t > 1).
+// G = sum_e gx_e; dL_ch += G.  (dr_{e'}^{t-1} = G - gx_{e'} is formed by the
+// adjoint check update that reads it: the edge gradients are then gathered
+// once and not scattered.)  Rows in CSC order, several in flight.
 template <int W>
-__global__ void __launch_bounds__(kBlock) kw_var_bwd(WArgs a, const float *gx, float *glch, float *gr_prev) {
+__global__ void __launch_bounds__(kBlock) kw_var_bwd(WArgs a, const float *gx, float *glch, float *G) {
     constexpr int TPC = W / kK;
+    constexpr int kRound = 8;
     const int slab = blockIdx.y;
     const int64_t lt = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     const int32_t v = static_cast<int32_t>(lt / TPC);
     if (v >= a.n_core) return;
     const int lane0 = static_cast<int>(lt % TPC) * kK;
-    const size_t ebase = static_cast<size_t>(slab) * a.e_core;
-    float4 G = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int32_t j = a.vptr[v]; j < a.vptr[v + 1]; ++j) {
-        const float4 g = ldf4(gx + (ebase + a.vedge[j]) * W + lane0);
-        G.x += g.x; G.y += g.y; G.z += g.z; G.w += g.w;
+    const float *row = gx + static_cast<size_t>(slab) * a.e_core * W + lane0;
+    const size_t o0 = (static_cast<size_t>(slab) * a.n_core + v) * W + lane0;
+    float4 o = *reinterpret_cast<float4 *>(glch + o0);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int32_t j1 = __ldg(a.vptr + v + 1);
+    for (int32_t j = __ldg(a.vptr + v); j < j1; j += kRound) {
+        float4 g[kRound];
+#pragma unroll
+        for (int k = 0; k < kRound; ++k)
+            if (j + k < j1) g[k] = ldf4(row + static_cast<size_t>(__ldg(a.vedge + j + k)) * W);
+#pragma unroll
+        for (int k = 0; k < kRound; ++k)
+            if (j + k < j1) { s.x += g[k].x; s.y += g[k].y; s.z += g[k].z; s.w += g[k].w; }
     }
-    float *gl = glch + (static_cast<size_t>(slab) * a.n_core + v) * W + lane0;
-    float4 o = *reinterpret_cast<float4 *>(gl);
-    o.x += G.x; o.y += G.y; o.z += G.z; o.w += G.w;
-    *reinterpret_cast<float4 *>(gl) = o;
-    if (gr_prev) {
-        for (int32_t j = a.vptr[v]; j < a.vptr[v + 1]; ++j) {
-            const size_t idx = (ebase + a.vedge[j]) * W + lane0;
-            const float4 g = ldf4(gx + idx);
-            *reinterpret_cast<float4 *>(gr_prev + idx) = make_float4(G.x - g.x, G.y - g.y, G.z - g.z, G.w - g.w);
-        }
-    }
-}
-
-// dloss/dr^T of core edge e = dloss/dL_v(e) (the posterior is L_ch + sum r^T).
-template <int W>
-__global__ void __launch_bounds__(kBlock) kw_grad_edges(WArgs a, const float *gl_core, float *gr) {
-    constexpr int TPC = W / kK;
-    const int slab = blockIdx.y;
-    const int64_t lt = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int32_t v = static_cast<int32_t>(lt / TPC);
-    if (v >= a.n_core) return;
-    const int lane0 = static_cast<int>(lt % TPC) * kK;
-    const float4 g = ldf4(gl_core + (static_cast<size_t>(slab) * a.n_core + v) * W + lane0);
-    for (int32_t j = a.vptr[v]; j < a.vptr[v + 1]; ++j)
-        *reinterpret_cast<float4 *>(gr + ((static_cast<size_t>(slab) * a.e_core + a.vedge[j]) * W + lane0)) = g;
+    o.x += s.x; o.y += s.y; o.z += s.z; o.w += s.w;
+    *reinterpret_cast<float4 *>(glch + o0) = o;
+    *reinterpret_cast<float4 *>(G + o0) = s;
 }
 
 // Natural [B][n] -> interleaved core / degree-1 arrays (32 VNs x W codewords per block).
 template <int W>
 __global__ void __launch_bounds__(kBlock) kw_interleave(const float *in, const int32_t *unit, int32_t n_vn,
                                                         int32_t n_core, int32_t n_deg1, int32_t batch, float *core,
-                                                        float *deg1, float *deg1_copy) {
+                                                        float *core_copy, float *deg1, float *deg1_copy) {
     __shared__ float tile[W][33];
     const int slab = blockIdx.y;
     const int32_t j0 = blockIdx.x * 32;
@@ -361,7 +674,9 @@ __global__ void __launch_bounds__(kBlock) kw_interleave(const float *in, const i
         const int32_t u = unit[j];
         const float v = tile[w][jj];
         if (u < n_core) {
-            core[(static_cast<size_t>(slab) * n_core + u) * W + w] = v;
+            const size_t o = (static_cast<size_t>(slab) * n_core + u) * W + w;
+            core[o] = v;
+            core_copy[o] = v;
         } else {
             const size_t o = (static_cast<size_t>(slab) * n_deg1 + (u - n_core)) * W + w;
             deg1[o] = v;
@@ -411,11 +726,13 @@ __global__ void __launch_bounds__(kBlock) kw_deinterleave(const float *core, con
 
 // Sum over the per-block partials of each weight type in a fixed order
 // (strided over the threads, then a shared-memory tree), so the result does
-// not depend on scheduling.
+// not depend on scheduling.  One block per iteration (row block y of gwp).
 constexpr int kReduceThreads = 256;
 __global__ void __launch_bounds__(kReduceThreads) kw_reduce_dw(const float *gwp, int blocks, int n_types,
-                                                               float *dw_row) {
+                                                               float *dw) {
     __shared__ float part[kReduceThreads];
+    gwp += static_cast<size_t>(blockIdx.x) * blocks * n_types;
+    float *dw_row = dw + static_cast<size_t>(blockIdx.x) * n_types;
     for (int k = 0; k < n_types; ++k) {
         float v = 0.f;
         for (int b = threadIdx.x; b < blocks; b += kReduceThreads) v += gwp[static_cast<size_t>(b) * n_types + k];
@@ -438,7 +755,7 @@ struct mld_tape {
     float *w = nullptr;                 // [T][n_types]
     std::vector<float *> ckpt;          // r^{k}, r^{2k}, ... (r^0 = 0)
     float *seg_r = nullptr, *seg_lv = nullptr;  // k message / posterior arrays
-    float *gr = nullptr, *gx = nullptr;          // edge gradients
+    float *G = nullptr, *gx = nullptr;           // VN sums and edge gradients
     float *glch = nullptr, *glch1 = nullptr, *gd1 = nullptr;
     float *gwp = nullptr;
     int gwp_blocks = 0;
@@ -458,7 +775,7 @@ void tape_free(mld_tape *t) {
     dfree(t->dw);
     dfree(t->w);
     for (float *&p : t->ckpt) dfree(p);
-    dfree(t->seg_r); dfree(t->seg_lv); dfree(t->gr); dfree(t->gx);
+    dfree(t->seg_r); dfree(t->seg_lv); dfree(t->G); dfree(t->gx);
     dfree(t->glch); dfree(t->glch1); dfree(t->gd1); dfree(t->gwp);
     delete t;
 }
@@ -501,32 +818,19 @@ WArgs wargs(const mld_decoder *d, const float *w, int n_types) {
                  h.n_cn, h.n_core, h.n_deg1, h.e_core, n_types, d->sbits, d->lch, d->lch1, w, d->lmax, d->amin};
 }
 
-// Forward iterations t = t_begin+1 .. t_end on messages r / posteriors lv.
+// Variable update: posteriors lv from messages r.
 template <int W>
-int forward_iters(mld_decoder *d, const WArgs &wa, float *r, float *lv, int t_begin, int t_end, int T, int slabs,
-                  cudaStream_t st, mld_tape *tape, float *seg_r, float *seg_lv) {
+int wbp_posteriors(mld_decoder *d, const float *r, float *lv, int slabs, cudaStream_t st) {
     const mld::HostGraph &h = d->g->h;
-    const size_t rsz = static_cast<size_t>(slabs) * h.e_core * W;
-    const size_t lsz = static_cast<size_t>(slabs) * h.n_core * W;
+    if (h.n_core == 0) return MLD_OK;
     VnArgs va{d->g->vptr, d->g->vedge, h.n_core, h.e_core, r, d->lch, lv, d->hb_core, d->done, 0, 0};
-    for (int t = t_begin + 1; t <= t_end; ++t) {
-        if (seg_r) {  // keep r^{t-1}, L^{t-1} for the adjoint of iteration t
-            MLD_CUDA(cudaMemcpyAsync(seg_r + (t - 1 - t_begin) * rsz, r, rsz * sizeof(float), cudaMemcpyDeviceToDevice, st));
-            MLD_CUDA(cudaMemcpyAsync(seg_lv + (t - 1 - t_begin) * lsz, lv, lsz * sizeof(float),
-                                     cudaMemcpyDeviceToDevice, st));
-        }
-        for (const mld::ClassLaunch &cl : d->g->launches[W == 8 ? 0 : (W == 16 ? 1 : (W == 32 ? 2 : 3))]) {
-            launch_check_fwd<W>(wa, cl, r, lv, d->post1, t, t == T ? 1 : 0, slabs, st);
-            MLD_LAUNCHED("kw_check_fwd");
-        }
-        if (h.n_core > 0) {
-            k_var_update<float, W><<<dim3(grid_x(static_cast<int64_t>(h.n_core) * (W / kVnLanes)), slabs), kBlock, 0, st>>>(va);
-            MLD_LAUNCHED("k_var_update");
-        }
-        if (tape && !seg_r && t % tape->k == 0 && t < T)
-            MLD_CUDA(cudaMemcpyAsync(tape->ckpt[t / tape->k - 1], r, rsz * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    }
+    k_var_update<float, W><<<dim3(grid_x(static_cast<int64_t>(h.n_core) * (W / kVnLanes)), slabs), kBlock, 0, st>>>(va);
+    MLD_LAUNCHED("k_var_update");
     return MLD_OK;
+}
+
+const std::vector<mld::ClassLaunch> &width_launches(const mld_decoder *d, int W) {
+    return d->g->launches[W == 8 ? 0 : (W == 16 ? 1 : (W == 32 ? 2 : 3))];
 }
 
 template <int W>
@@ -534,20 +838,30 @@ int wbp_forward_w(mld_decoder *d, const float *llr, const uint8_t *syn, int32_t 
                   const float *w, int n_types, float *soft, cudaStream_t st) {
     const mld::HostGraph &h = d->g->h;
     const int slabs = (batch + W - 1) / W;
-    const size_t rsz = static_cast<size_t>(slabs) * h.e_core * W;
     // weighted BP works in nats: no scaling on entry or exit
     InArgs ia{llr, nullptr, d->g->unit, h.n_vn, h.n_core, h.n_deg1, batch, d->lmax, 1.f, d->lmax, d->amin,
               d->lch, d->Lv, d->lch1, d->post1, d->phi1};
-    const PrologueArgs pa{ia, syn, d->g->cint, d->sbits, h.n_cn, (h.n_vn + 31) / 32, static_cast<uint4 *>(d->r),
-                          rsz * sizeof(float) / 16};
+    // (the first iteration reads no messages: nothing to clear)
+    const PrologueArgs pa{ia, syn, d->g->cint, d->sbits, h.n_cn, (h.n_vn + 31) / 32, nullptr, 0};
     if (h.n_vn > 0 || h.n_cn > 0) {
         k_prologue<W, kFitNat><<<dim3(pa.in_tiles + (h.n_cn + 31) / 32, slabs), kBlock, 0, st>>>(pa);
         MLD_LAUNCHED("k_prologue");
     }
     const WArgs wa = wargs(d, w, n_types);
-    auto iters = [&](cudaStream_t s2) {
-        return forward_iters<W>(d, wa, static_cast<float *>(d->r), d->Lv, 0, T, T, slabs, s2, tape, nullptr,
-                                nullptr);
+    auto iters = [&](cudaStream_t s2) -> int {
+        // an iteration whose messages the tape keeps writes them there
+        const WbpClasses classes = wbp_classes(width_launches(d, W));
+        const float *r_in = nullptr;
+        for (int t = 1; t <= T; ++t) {
+            const bool keep = tape && t % tape->k == 0 && t < T;
+            float *r_out = keep ? tape->ckpt[t / tape->k - 1] : static_cast<float *>(d->r);
+            launch_fwd<W>(wa, classes, r_in, r_out, d->Lv, d->post1, t, t == T ? 1 : 0, slabs, s2);
+            MLD_LAUNCHED("kw_fwd");
+            const int q = wbp_posteriors<W>(d, r_out, d->Lv, slabs, s2);
+            if (q != MLD_OK) return q;
+            r_in = r_out;
+        }
+        return MLD_OK;
     };
     // with a tape every buffer the iterations touch is fixed for the tape's
     // life (the weights were copied into it), so they run as a graph
@@ -573,68 +887,58 @@ int wbp_backward_w(mld_tape *tp, const float *dsoft, float *dw, float *dllr, cud
     const size_t dsz = static_cast<size_t>(slabs) * h.n_deg1 * W;
     const WArgs wa = wargs(d, tp->w, tp->n_types);
     const dim3 vgrid(grid_x(static_cast<int64_t>(h.n_core) * TPC), slabs);
-    const std::vector<mld::ClassLaunch> &classes = d->g->launches[W == 8 ? 0 : (W == 16 ? 1 : (W == 32 ? 2 : 3))];
-    int32_t parts = 0;  // block partials of one adjoint check pass
-    for (const mld::ClassLaunch &cl : classes) parts += cl.blocks * slabs;
+    const WbpClasses classes = wbp_classes(width_launches(d, W));
+    const int32_t parts = classes.parts * slabs;  // block partials of one adjoint check pass
 
     // dloss/dL^T: into dL_ch (the posterior is L_ch + sum r^T) and onto r^T
     if (lsz) MLD_CUDA(cudaMemsetAsync(tp->glch, 0, lsz * sizeof(float), st));
     if (dsz) MLD_CUDA(cudaMemsetAsync(tp->glch1, 0, dsz * sizeof(float), st));
     if (h.n_vn > 0) {
         kw_interleave<W><<<dim3((h.n_vn + 31) / 32, slabs), kBlock, 0, st>>>(
-            dsoft, d->g->unit, h.n_vn, h.n_core, h.n_deg1, tp->batch, tp->glch, tp->glch1, tp->gd1);
+            dsoft, d->g->unit, h.n_vn, h.n_core, h.n_deg1, tp->batch, tp->glch, tp->G, tp->glch1, tp->gd1);
         MLD_LAUNCHED("kw_interleave");
     }
     // from dL^T on, every buffer is the tape's or the decoder's: the
     // segments run as a graph (dw into the tape, then copied out)
     auto segments = [&](cudaStream_t s2) -> int {
-        if (h.n_core > 0) {
-            kw_grad_edges<W><<<vgrid, kBlock, 0, s2>>>(wa, tp->glch, tp->gr);
-            MLD_LAUNCHED("kw_grad_edges");
-        }
-        float *r = static_cast<float *>(d->r);
+        // dloss/dr^T of core edge e is dloss/dL_v(e): G holds it, no gx yet
         for (int t0 = ((T - 1) / K) * K; t0 >= 0; t0 -= K) {
             const int t1 = std::min(t0 + K, T);
-            // recompute r^{t0} .. r^{t1-1} and L^{t0} .. L^{t1-1}
-            if (t0 == 0) {
-                if (rsz) MLD_CUDA(cudaMemsetAsync(r, 0, rsz * sizeof(float), s2));
+            // recompute r^{t0+1} .. r^{t1-1} and L^{t0} .. L^{t1-1}
+            auto seg_r = [&](int t) -> const float * {
+                return t == 0 ? nullptr : t == t0 ? tp->ckpt[t0 / K - 1] : tp->seg_r + static_cast<size_t>(t - t0 - 1) * rsz;
+            };
+            auto seg_lv = [&](int t) { return tp->seg_lv + static_cast<size_t>(t - t0) * lsz; };
+            if (t0 == 0) {  // no messages: the posteriors are the channel values
+                if (lsz)
+                    MLD_CUDA(cudaMemcpyAsync(seg_lv(0), d->lch, lsz * sizeof(float), cudaMemcpyDeviceToDevice, s2));
             } else {
-                MLD_CUDA(cudaMemcpyAsync(r, tp->ckpt[t0 / K - 1], rsz * sizeof(float), cudaMemcpyDeviceToDevice, s2));
+                const int q = wbp_posteriors<W>(d, seg_r(t0), seg_lv(t0), slabs, s2);
+                if (q != MLD_OK) return q;
             }
-            if (h.n_core > 0) {
-                VnArgs va{d->g->vptr, d->g->vedge, h.n_core, h.e_core, r, d->lch, d->Lv, d->hb_core, d->done, 0, 0};
-                k_var_update<float, W><<<dim3(grid_x(static_cast<int64_t>(h.n_core) * (W / kVnLanes)), slabs), kBlock, 0, s2>>>(va);
-                MLD_LAUNCHED("k_var_update");
+            for (int t = t0 + 1; t < t1; ++t) {
+                float *out = const_cast<float *>(seg_r(t));
+                launch_fwd<W>(wa, classes, seg_r(t - 1), out, seg_lv(t - 1), d->post1, t, 0, slabs, s2);
+                MLD_LAUNCHED("kw_fwd");
+                const int q = wbp_posteriors<W>(d, out, seg_lv(t), slabs, s2);
+                if (q != MLD_OK) return q;
             }
-            int s = forward_iters<W>(d, wa, r, d->Lv, t0, t1 - 1, T, slabs, s2, tp, tp->seg_r, tp->seg_lv);
-            if (s != MLD_OK) return s;
-            // r^{t1-1}, L^{t1-1} are now in r / d->Lv; store them as the last segment entry
-            MLD_CUDA(cudaMemcpyAsync(tp->seg_r + (t1 - 1 - t0) * rsz, r, rsz * sizeof(float), cudaMemcpyDeviceToDevice, s2));
-            MLD_CUDA(cudaMemcpyAsync(tp->seg_lv + (t1 - 1 - t0) * lsz, d->Lv, lsz * sizeof(float),
-                                     cudaMemcpyDeviceToDevice, s2));
             for (int t = t1; t > t0; --t) {
-                const float *rp = tp->seg_r + (t - 1 - t0) * rsz;
-                const float *lvp = tp->seg_lv + (t - 1 - t0) * lsz;
-                if (parts > 0) {
-                    int32_t part0 = 0;
-                    for (const mld::ClassLaunch &cl : classes) {
-                        launch_check_bwd<W>(wa, cl, rp, lvp, tp->gr, t == T ? tp->gd1 : nullptr, tp->gx, tp->glch1,
-                                            tp->gwp, t, slabs, part0, s2);
-                        MLD_LAUNCHED("kw_check_bwd");
-                        part0 += cl.blocks * slabs;
-                    }
-                    kw_reduce_dw<<<1, kReduceThreads, 0, s2>>>(tp->gwp, parts, tp->n_types,
-                                                               tp->dw + static_cast<size_t>(t - 1) * tp->n_types);
-                    MLD_LAUNCHED("kw_reduce_dw");
-                } else {
-                    MLD_CUDA(cudaMemsetAsync(tp->dw + static_cast<size_t>(t - 1) * tp->n_types, 0,
-                                             sizeof(float) * tp->n_types, s2));
-                }
+                launch_bwd<W>(wa, classes, seg_r(t - 1), seg_lv(t - 1), tp->G, t < T ? 1 : 0, tp->gx,
+                              t == T ? tp->gd1 : nullptr, tp->glch1,
+                              tp->gwp + static_cast<size_t>(t - 1) * parts * tp->n_types, t, slabs, s2);
+                MLD_LAUNCHED("kw_bwd");
                 if (h.n_core > 0) {
-                    kw_var_bwd<W><<<vgrid, kBlock, 0, s2>>>(wa, tp->gx, tp->glch, t > 1 ? tp->gr : nullptr);
+                    kw_var_bwd<W><<<vgrid, kBlock, 0, s2>>>(wa, tp->gx, tp->glch, tp->G);
                     MLD_LAUNCHED("kw_var_bwd");
                 }
             }
+        }
+        if (parts > 0) {
+            kw_reduce_dw<<<T, kReduceThreads, 0, s2>>>(tp->gwp, parts, tp->n_types, tp->dw);
+            MLD_LAUNCHED("kw_reduce_dw");
+        } else {
+            MLD_CUDA(cudaMemsetAsync(tp->dw, 0, sizeof(float) * T * tp->n_types, s2));
         }
         return MLD_OK;
     };
@@ -733,9 +1037,9 @@ int mld_wbp_forward(mld_decoder *d, const float *llr, const uint8_t *syndrome, i
             s = talloc(&p, rsz);
             tp->ckpt.push_back(p);
         }
-        if (s == MLD_OK) s = talloc(&tp->seg_r, rsz * tp->k);
+        if (s == MLD_OK) s = talloc(&tp->seg_r, rsz * (tp->k - 1));
         if (s == MLD_OK) s = talloc(&tp->seg_lv, lsz * tp->k);
-        if (s == MLD_OK) s = talloc(&tp->gr, rsz);
+        if (s == MLD_OK) s = talloc(&tp->G, lsz);
         if (s == MLD_OK) s = talloc(&tp->gx, rsz);
         if (s == MLD_OK) s = talloc(&tp->glch, lsz);
         if (s == MLD_OK) s = talloc(&tp->glch1, dsz);
@@ -743,7 +1047,7 @@ int mld_wbp_forward(mld_decoder *d, const float *llr, const uint8_t *syndrome, i
         tp->gwp_blocks = 0;
         for (const mld::ClassLaunch &cl : d->g->launches[W == 8 ? 0 : (W == 16 ? 1 : (W == 32 ? 2 : 3))])
             tp->gwp_blocks += cl.blocks * slabs;
-        if (s == MLD_OK) s = talloc(&tp->gwp, static_cast<size_t>(std::max(1, tp->gwp_blocks)) * n_types);
+        if (s == MLD_OK) s = talloc(&tp->gwp, static_cast<size_t>(std::max(1, tp->gwp_blocks)) * T * n_types);
         if (s == MLD_OK) {
             cudaError_t e = cudaMemcpyAsync(tp->w, w, sizeof(float) * T * n_types, cudaMemcpyDeviceToDevice, st);
             if (e != cudaSuccess) s = cuda_fail(e, "wbp_forward: copy weights");
