@@ -77,7 +77,11 @@ __device__ __forceinline__ float2 pair_of(const float4 &v, int p) {
 // Check kernels of the register classes: one launch covers every class of the
 // graph, a block finds its class in a table and runs the body of its shape
 // (DC core edges, DD degree-1 VNs), with every operand of a check requested
-// before any arithmetic and the arithmetic two codewords at a time.
+// before any arithmetic and the arithmetic two codewords at a time.  Bound by
+// latency at the few blocks their registers allow: n = 10^5, 16 codewords, T =
+// 20, training step 2.38 ms at 4 / 3 blocks per SM (forward / adjoint, no
+// spills), 2.22 ms at 6 / 4, 2.33 ms at 8 / 5 (4.95 ms with the runtime-degree
+// kernels, one launch per class).
 // ---------------------------------------------------------------------------
 constexpr int kMaxTable = 16;
 struct ClassTable {
@@ -288,7 +292,7 @@ __device__ __forceinline__ bool table_check(const ClassTable &tb, int &k, int32_
     X(0, 1) X(1, 1) X(2, 1) X(3, 1) X(4, 1) X(5, 1) X(6, 1) X(7, 1)
 
 template <int W>
-__global__ void __launch_bounds__(kBlock, 4) kw_fwd(WArgs a, ClassTable tb, const float *r_in, float *r_out,
+__global__ void __launch_bounds__(kBlock, 6) kw_fwd(WArgs a, ClassTable tb, const float *r_in, float *r_out,
                                                     const float *lv, float *post1, int t, int last) {
     int k, lane0;
     int32_t j;
@@ -325,7 +329,7 @@ __device__ __forceinline__ void block_weight_sums(const float (&gw)[kMaxTypes], 
 }
 
 template <int W>
-__global__ void __launch_bounds__(kBlock, 3) kw_bwd(WArgs a, ClassTable tb, const float *rp, const float *lvp,
+__global__ void __launch_bounds__(kBlock, 4) kw_bwd(WArgs a, ClassTable tb, const float *rp, const float *lvp,
                                                     const float *G, int gx_used, float *gx, const float *gd1,
                                                     float *glch1, float *gwp, int t) {
     float gw[kMaxTypes];
