@@ -16,6 +16,7 @@
 // start.
 #include <map>
 #include <tuple>
+#include <type_traits>
 
 #include "kernels.cuh"
 
@@ -43,10 +44,16 @@ struct Seg {
     ClassLaunch cl;
 };
 
+// The segment of this block (segments are sorted by their first block, the
+// first one's is 0): every lane looks at one.
 __device__ __forceinline__ int find_seg(const Seg *segs, int nseg) {
-    int k = 0;
-    while (k + 1 < nseg && static_cast<int32_t>(blockIdx.x) >= segs[k + 1].block0) ++k;
-    return k;
+    const int lane = threadIdx.x & 31;
+    int below = 0;
+    for (int i0 = 0; i0 < nseg; i0 += 32) {
+        const int i = i0 + lane;
+        below += __popc(__ballot_sync(0xFFFFFFFFu, i < nseg && segs[i].block0 <= static_cast<int32_t>(blockIdx.x)));
+    }
+    return below - 1;
 }
 
 // Check arguments of job j in an iteration of the given parity (its degree-1
@@ -71,6 +78,35 @@ __global__ void __launch_bounds__(kBlock, (kCheckBlocksPerSm<DC + DD>))
     extern __shared__ __align__(128) unsigned char smem[];
     check_class_body<MsgT, W, DC, DD, PASS>(
         a, sg.cl, static_cast<int64_t>(local % sg.bps) * blockDim.x + threadIdx.x, sg.bps, slab, smem);
+}
+
+// Shapes of up to six terms share one launch: the graph's small classes (a few
+// checks to a few percent) then cost blocks instead of launches, of which a
+// plan of three rates has eight per width and iteration.
+#define MLD_MERGED_SHAPES(X)                                                           \
+    X(1, 0) X(2, 0) X(3, 0) X(4, 0) X(5, 0) X(6, 0)                                     \
+    X(0, 1) X(1, 1) X(2, 1) X(3, 1) X(4, 1) X(5, 1)
+template <typename MsgT>
+constexpr int kMergedSmem = RingShape<MsgT, 6, 0>::kBytes > RingShape<MsgT, 5, 1>::kBytes ? RingShape<MsgT, 6, 0>::kBytes
+                                                                                         : RingShape<MsgT, 5, 1>::kBytes;
+
+template <typename MsgT, int W, int PASS>
+__global__ void __launch_bounds__(kBlock, (kCheckBlocksPerSm<6>))
+    km_check_merged(const JobDev *jobs, const Seg *segs, int nseg, int parity) {
+    const Seg sg = segs[find_seg(segs, nseg)];
+    const CnArgs a = job_cn<W>(jobs[sg.job], sg, parity);
+    const int local = blockIdx.x - sg.block0;
+    const int slab = local / sg.bps;
+    if (a.et && slab_all_done<W>(a.done, slab)) return;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int64_t t0 = static_cast<int64_t>(local % sg.bps) * blockDim.x + threadIdx.x;
+    switch (sg.cl.dc * 2 + (sg.cl.deg - sg.cl.dc)) {
+#define X(DC, DD) \
+    case (DC) * 2 + (DD): check_class_body<MsgT, W, DC, DD, PASS>(a, sg.cl, t0, sg.bps, slab, smem); break;
+        MLD_MERGED_SHAPES(X)
+#undef X
+        default: break;
+    }
 }
 
 template <typename MsgT, int W>
@@ -220,24 +256,26 @@ template <typename MsgT, int W>
 void launch_check_op(const mld_plan *p, const Op &op, cudaStream_t st) {
     const JobDev *J = p->d_jobs;
     const Seg *S = p->d_segs + op.seg0;
+    auto run = [&](auto bytes, auto kernel) {
+        allow_smem<decltype(bytes)::value>(kernel);
+        kernel<<<op.blocks, kBlock, decltype(bytes)::value, st>>>(J, S, op.nseg, op.parity);
+    };
+    if (op.dc == 0) {
+        const std::integral_constant<int, kMergedSmem<MsgT>> sm;
+        if (op.pass == kPassHard) run(sm, km_check_merged<MsgT, W, kPassHard>);
+        else if (op.pass == kPassPlain) run(sm, km_check_merged<MsgT, W, kPassPlain>);
+        else run(sm, km_check_merged<MsgT, W, kPassFull>);
+        return;
+    }
 #define MLD_CASE(DCV, DDV)                                                                          \
     if (op.dc == (DCV) && op.dd == (DDV)) {                                                         \
-        constexpr int sm = RingShape<MsgT, DCV, DDV>::kBytes;                                      \
-        if (op.pass == kPassHard) allow_smem<sm>(km_check<MsgT, W, DCV, DDV, kPassHard>);           \
-        else if (op.pass == kPassPlain) allow_smem<sm>(km_check<MsgT, W, DCV, DDV, kPassPlain>);    \
-        else allow_smem<sm>(km_check<MsgT, W, DCV, DDV, kPassFull>);                                \
-        if (op.pass == kPassHard)                                                                   \
-            km_check<MsgT, W, DCV, DDV, kPassHard><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.parity); \
-        else if (op.pass == kPassPlain)                                                             \
-            km_check<MsgT, W, DCV, DDV, kPassPlain><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.parity); \
-        else                                                                                        \
-            km_check<MsgT, W, DCV, DDV, kPassFull><<<op.blocks, kBlock, sm, st>>>(J, S, op.nseg, op.parity); \
+        const std::integral_constant<int, RingShape<MsgT, DCV, DDV>::kBytes> sm;                    \
+        if (op.pass == kPassHard) run(sm, km_check<MsgT, W, DCV, DDV, kPassHard>);                  \
+        else if (op.pass == kPassPlain) run(sm, km_check<MsgT, W, DCV, DDV, kPassPlain>);           \
+        else run(sm, km_check<MsgT, W, DCV, DDV, kPassFull>);                                       \
         return;                                                                                     \
     }
-    MLD_CASE(1, 0) MLD_CASE(2, 0) MLD_CASE(3, 0) MLD_CASE(4, 0)
-    MLD_CASE(5, 0) MLD_CASE(6, 0) MLD_CASE(7, 0) MLD_CASE(8, 0)
-    MLD_CASE(0, 1) MLD_CASE(1, 1) MLD_CASE(2, 1) MLD_CASE(3, 1)
-    MLD_CASE(4, 1) MLD_CASE(5, 1) MLD_CASE(6, 1) MLD_CASE(7, 1)
+    MLD_CASE(7, 0) MLD_CASE(8, 0) MLD_CASE(6, 1) MLD_CASE(7, 1)
 #undef MLD_CASE
     km_check_irregular<MsgT, W><<<op.blocks, kBlock, 0, st>>>(J, S, op.nseg, op.parity);
 }
@@ -527,7 +565,9 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
                 const int pass = !regular ? kPassFull : (et && !jobs[j].post_out) ? kPassHard : fl ? kPassFull : kPassPlain;
                 Seg s = seg(j, regular ? class_blocks(cl, sm_count) : cl.blocks, jd[j].slabs, fl);
                 s.cl = cl;
-                groups[Key{kOpCheck, half, jd[j].W, regular ? cl.dc : -1, regular ? dd : -1, pass}].push_back(s);
+                const bool merged = regular && cl.deg <= 6;
+                groups[Key{kOpCheck, half, jd[j].W, merged ? 0 : regular ? cl.dc : -1, merged ? 0 : regular ? dd : -1, pass}]
+                    .push_back(s);
             }
         }
         flush(groups, l, parity);
