@@ -30,6 +30,12 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
     d->sample_now = true;
     InArgs ia{in, sigma, g->unit, h.n_vn, h.n_core, h.n_deg1, batch, d->lmax, d->scale_in, d->lmax_i, d->amin_i,
               d->lch, acc_mode ? acc_of(0) : d->Lv, d->lch1, d->post1, d->phi1};
+    // What only some kernels read: a decode that iterates writes the degree-1
+    // posteriors before it reads them, and the decisions-only form of the
+    // register classes needs no degree-1 channel LLRs (205 MB each at rate 0.1,
+    // n = 10^6, 64 codewords).
+    if (iters > 0) ia.post1 = nullptr;
+    if (iters > 0 && et && !post && g->acc_ok && d->check_rule == MLD_CHECK_SUM_PRODUCT) ia.lch1 = nullptr;
     const PrologueArgs pa{ia, syn, g->cint, d->sbits, h.n_cn, (h.n_vn + 31) / 32, static_cast<uint4 *>(d->r),
                           static_cast<size_t>(slabs) * h.e_core * W * sizeof(MsgT) / 16};
     if (h.n_vn > 0 || h.n_cn > 0) {
@@ -51,8 +57,8 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
         const bool hard = et && !post;
         int32_t *io = out_dev ? iters_out : nullptr;
         uint8_t *co = out_dev ? conv_out : nullptr;
-        if constexpr (IsHalf<MsgT>::value) small = mld::small_decode_f16(d, W, batch, iters, et, hard, io, co, sm_count, st);
-        else small = mld::small_decode_f32(d, W, batch, iters, et, hard, io, co, sm_count, st);
+        if constexpr (IsHalf<MsgT>::value) small = mld::small_decode_f16(d, W, batch, iters, et, hard, io, co, sm_count, st, post != nullptr);
+        else small = mld::small_decode_f32(d, W, batch, iters, et, hard, io, co, sm_count, st, post != nullptr);
     }
     if (!small) MLD_CUDA(cudaMemsetAsync(d->done, 0, sizeof(uint32_t) * slabs * DW, st));
 
@@ -65,6 +71,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
               d->lmax_i, d->amin_i, 0, et ? 1 : 0};
     ca.status = d->status;
     ca.stall_test = d->stall_test;
+    if (!et && !post) ca.post1 = nullptr;  // nothing reads the degree-1 posteriors
     ca.rule = d->check_rule == MLD_CHECK_MIN_SUM ? kRuleMinSum : kRuleSumProduct;
     ca.ms_off = d->ms_off_i;
     // early termination without soft output: degree-1 decisions only (a

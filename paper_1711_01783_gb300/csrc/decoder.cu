@@ -91,7 +91,7 @@ void decoder_free(mld_decoder *d) {
     if (d->cap) cudaStreamDestroy(d->cap);
     d->cap = nullptr;
     dfree(d->lctr);
-    dfree(d->bar);
+    d->bar = nullptr;  // (part of the status allocation)
 }
 
 // The device address of a page-locked, mapped host buffer; null for any
@@ -438,7 +438,8 @@ int mld_decoder_create(const mld_graph *g, const mld_opts *opts, mld_decoder **o
     if (s == MLD_OK) s = dalloc(&d->fail, 2 * S * DW);  // two buffers (iteration parity) for plans
     if (s == MLD_OK) s = dalloc(&d->iters, S * W);
     if (s == MLD_OK) s = dalloc(&d->conv, S * W);
-    if (s == MLD_OK) s = dalloc(&d->status, 4);
+    if (s == MLD_OK) s = dalloc(&d->status, 8);  // status word and its record, grid barrier
+    if (s == MLD_OK) d->bar = reinterpret_cast<uint32_t *>(d->status + 4);
     if (s == MLD_OK && d->checked) {
         cudaError_t ce = cudaHostAlloc(reinterpret_cast<void **>(&d->status_host), 4 * sizeof(int32_t),
                                        cudaHostAllocDefault);
@@ -453,7 +454,6 @@ int mld_decoder_create(const mld_graph *g, const mld_opts *opts, mld_decoder **o
     if (s == MLD_OK) s = dalloc(&d->syn_stage, static_cast<size_t>(d->max_batch) * h.n_cn);
     if (s == MLD_OK) s = dalloc(&d->bits_stage, nb);
     if (s == MLD_OK) s = dalloc(&d->lctr, 2);
-    if (s == MLD_OK) s = dalloc(&d->bar, 3);
     if (s == MLD_OK) {
         cudaError_t ce = cudaStreamCreateWithFlags(&d->cap, cudaStreamNonBlocking);
         if (ce != cudaSuccess) s = cuda_fail(ce, "decoder_create: capture stream");
@@ -465,8 +465,7 @@ int mld_decoder_create(const mld_graph *g, const mld_opts *opts, mld_decoder **o
         if (ce != cudaSuccess) s = cuda_fail(ce, "decoder_create: side stream");
     }
     if (s == MLD_OK) {
-        cudaError_t e2 = cudaMemset(d->status, 0, 4 * sizeof(int32_t));
-        if (e2 == cudaSuccess) e2 = cudaMemset(d->bar, 0, 3 * sizeof(uint32_t));
+        cudaError_t e2 = cudaMemset(d->status, 0, 8 * sizeof(int32_t));
         if (e2 != cudaSuccess) s = cuda_fail(e2, "cudaMemset");
     }
     if (s != MLD_OK) {

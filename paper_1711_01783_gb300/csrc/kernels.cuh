@@ -383,7 +383,7 @@ __device__ __forceinline__ void emit_deg1(const CnArgs &a, int slab, int slot, i
         const uint32_t oldnib = (static_cast<uint32_t>(*hb) >> (lane0 & 7)) & 0xFu;
         nib = (nib & ~donenib) | (oldnib & donenib);
     }
-    if (valid) *reinterpret_cast<float4 *>(a.post1 + base) = post;
+    if (valid && a.post1) *reinterpret_cast<float4 *>(a.post1 + base) = post;
     const uint32_t other = __shfl_xor_sync(pair_mask(), nib, 1);
     if (valid && (lane0 & 7) == 0) *hb = static_cast<uint8_t>(nib | (other << 4));
 }
@@ -1957,7 +1957,7 @@ struct InArgs {
     float lmax;           // clamp of the channel LLR, nats
     float scale;          // nats -> internal units (log2 e for decoding, 1 for weighted BP)
     float lmax_i, amin_i; // phi argument clamps in internal units
-    float *lch, *Lv, *lch1, *post1, *phi1;
+    float *lch, *Lv, *lch1, *post1, *phi1;  // (lch1, post1: null where no kernel of the call reads them)
 };
 
 // One tile of 32 natural VNs x W codewords of slab `slab`.
@@ -1993,8 +1993,8 @@ __device__ __forceinline__ void interleave_body(const InArgs &a, int tile_x, int
             a.Lv[o] = v;
         } else {
             const size_t o = (static_cast<size_t>(slab) * a.n_deg1 + (u - a.n_core)) * W + w;
-            a.lch1[o] = v;
-            a.post1[o] = v;
+            if (a.lch1) a.lch1[o] = v;
+            if (a.post1) a.post1[o] = v;
             // the degree-1 VN's message never changes: its phi term, with the
             // sign of the LLR, is formed once here for every check update
             const float f = phi_f<F>(clampf(fabsf(v), a.amin_i, a.lmax_i));
@@ -2263,9 +2263,9 @@ int run_decode_f32(mld_decoder *d, const float *in, const float *sigma, const ui
 // decode in one cooperative launch; false if it does not apply (nothing was
 // enqueued).  iters_out / conv_out: the caller's device arrays or null.
 bool small_decode_f16(mld_decoder *d, int W, int32_t batch, int32_t iters, bool et, bool hard1, int32_t *iters_out,
-                      uint8_t *conv_out, int sm_count, cudaStream_t st);
+                      uint8_t *conv_out, int sm_count, cudaStream_t st, bool soft);
 bool small_decode_f32(mld_decoder *d, int W, int32_t batch, int32_t iters, bool et, bool hard1, int32_t *iters_out,
-                      uint8_t *conv_out, int sm_count, cudaStream_t st);
+                      uint8_t *conv_out, int sm_count, cudaStream_t st, bool soft);
 // Sets the shared-memory carveout of the staged kernels that decode_f16.cu
 // launches (a function attribute belongs to one translation unit's kernel).
 cudaError_t prepare_staged_f16();

@@ -437,6 +437,12 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
         x.slabs = slabs;
         x.W = W;
         x.max_iters = jb.max_iters;
+        // (see the prologue of a single decode)
+        if (jb.max_iters > 0) {
+            x.in.post1 = nullptr;
+            if (et && !jb.post_out && d->g->acc_ok) x.in.lch1 = nullptr;
+            if (!et && !jb.post_out) x.cn.post1 = nullptr;
+        }
         jd.push_back(x);
         lmax_iters = std::max(lmax_iters, jb.max_iters);
     }

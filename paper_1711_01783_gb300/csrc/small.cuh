@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kSmallBlock, 1) k_small_decode(SmallArgs s) {
 // enqueued).
 template <typename MsgT, int W>
 bool launch_small(mld_decoder *d, int32_t batch, int32_t iters, bool et, bool hard1, int32_t *iters_out,
-                  uint8_t *conv_out, int sm_count, cudaStream_t st) {
+                  uint8_t *conv_out, int sm_count, cudaStream_t st, bool soft) {
     constexpr uint32_t TPC = W / kK;
     const mld::HostGraph &h = d->g->h;
     const mld_graph *g = d->g;
@@ -261,6 +261,7 @@ bool launch_small(mld_decoder *d, int32_t batch, int32_t iters, bool et, bool ha
     s.status = d->status;
     s.cn = CnArgs{g->cptr, g->col, g->dptr, h.n_cn, h.n_core, h.n_deg1, h.e_core, d->r, d->Lv, d->lch1, d->phi1,
                   d->post1, d->hb1, d->sbits, nullptr, d->lmax_i, d->amin_i, 0, et ? 1 : 0};
+    if (!et && !soft) s.cn.post1 = nullptr;
     s.vn = VnArgs{g->vptr, g->vedge, h.n_core, h.e_core, d->r, d->lch, d->Lv, d->hb_core, nullptr, 0, et ? 1 : 0};
     s.sy = SynArgs{g->cptr, g->col, g->dptr, h.n_cn, h.n_core, h.n_deg1, d->sbits, d->hb_core, d->hb1, d->fail,
                    nullptr, et ? 1 : 0, batch};
