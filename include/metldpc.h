@@ -47,7 +47,8 @@ extern "C" {
 #define MLD_ENOMEM   (-2)  /* host or device allocation failed                  */
 #define MLD_ECUDA    (-3)  /* a CUDA runtime call or kernel launch failed        */
 #define MLD_ETIMEOUT (-4)  /* a bounded device-side wait gave up (reported by
-                              mld_decode_status; see mld_opts.staging)        */
+                              mld_decode_status; see mld_opts.staging and
+                              mld_decode)                                     */
 #define MLD_EGRAPH   (-5)  /* malformed Tanner graph (index out of range, ...)   */
 
 /* ---- edge-message storage type (mld_opts.msg_dtype) ---------------------- */
@@ -254,8 +255,8 @@ int mld_peg_edges(int32_t n_vn, int32_t n_types, const int32_t *deg, int32_t n_c
  *                The result is kept for mld_decode_status.  A debugging aid
  *                for programs that may write stray device memory; plans do
  *                not check.
- *   staging    : MLD_STAGE_DIRECT (default): the check update reads its
- *                operands from device memory as it goes.  MLD_STAGE_BULK:
+ *   staging    : MLD_STAGE_DIRECT (default): every thread of the check update
+ *                copies its own operands one check ahead.  MLD_STAGE_BULK:
  *                where it applies (half messages at slab width 64,
  *                sum-product, flooding, MLD_VN_GATHER, checks of at most six
  *                terms with at most one degree-1 VN, and not the
@@ -265,7 +266,8 @@ int mld_peg_edges(int32_t n_vn, int32_t n_types, const int32_t *deg, int32_t n_c
  *                posterior row; MLD_STAGE_BULK_LSU: the same, with the
  *                posterior rows copied 16 bytes per thread by cp.async.
  *                Results are bit-identical to MLD_STAGE_DIRECT (and slower
- *                on GB300: the direct kernel is instruction-bound).  Waits
+ *                on GB300: the direct kernel requests its operands a check
+ *                ahead by itself).  Waits
  *                are bounded (2 s): a copy that never completes makes the
  *                decode's results invalid and mld_decode_status return
  *                MLD_ETIMEOUT.
@@ -320,7 +322,12 @@ int mld_decoder_destroy(mld_decoder *d);
  *                max_iters.
  * Errors: MLD_EINVAL (null pointer, batch > max_batch, negative max_iters,
  * unknown flag), MLD_ECUDA.  A device-detected error, if any, is reported
- * by mld_decode_status once the stream has completed. */
+ * by mld_decode_status once the stream has completed.
+ * Flooding sum-product gather decodes of small problems (up to ~600 000
+ * threads of a check update, checks of one to six core edges and at most one
+ * degree-1 VN) run their iterations in one cooperative launch whose blocks
+ * wait on one another at most 2 s; should such a wait run out, the results are
+ * invalid and mld_decode_status returns MLD_ETIMEOUT from then on. */
 int mld_decode(mld_decoder *d, const float *llr, const uint8_t *syndrome,
                int32_t batch, int32_t max_iters, uint32_t flags,
                uint8_t *bits_out, float *post_out, uint8_t *converged,
@@ -341,8 +348,9 @@ int mld_decode_y(mld_decoder *d, const float *y, const float *sigma,
  * the check of a decoder created with `checked` found the graph store
  * corrupted in its last decode call (array, index and value in
  * mld_last_error()), or MLD_ETIMEOUT when a staged check update
- * (MLD_STAGE_BULK) gave up waiting for a copy in some earlier call (sticky:
- * that decoder's later results are not to be trusted).  Reads the device
+ * (MLD_STAGE_BULK) gave up waiting for a copy, or a one-launch decode for its
+ * other blocks, in some earlier call (sticky: that decoder's later results are
+ * not to be trusted).  Reads the device
  * status word with a blocking copy; call after the stream is idle. */
 int mld_decode_status(mld_decoder *d);
 

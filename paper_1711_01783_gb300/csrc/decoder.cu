@@ -505,7 +505,8 @@ int mld_decode_status(mld_decoder *d) {
     cudaError_t e = cudaMemcpy(v, d->status, sizeof(v), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "decode_status");
     if (v[0] == MLD_ETIMEOUT)
-        return mld::fail(MLD_ETIMEOUT, "decode_status: a staged check update gave up waiting for a bulk copy");
+        return mld::fail(MLD_ETIMEOUT, "decode_status: a bounded wait on the device ran out (a staged check "
+                                       "update's bulk copy, or a grid barrier of a one-launch decode)");
     return v[0] == 0 ? MLD_OK : mld::fail(v[0], graph_fault_text(v));
 }
 

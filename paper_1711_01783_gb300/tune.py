@@ -13,8 +13,7 @@ termination to the variable-update variant as well: the gather pass or the
 accumulation of the new messages inside the check update (which wins with
 float messages and loses with half ones on GB300), over the slab widths each
 variant allows, and for half messages to the staged check update (operands
-brought into shared memory by bulk copies; slower on GB300, where the
-direct kernel is instruction-bound).  Plans keep the gather, so they use
+brought into shared memory by block-wide bulk copies; slower on GB300).  Plans keep the gather, so they use
 ``SlabWidthTuner``.
 """
 from __future__ import annotations

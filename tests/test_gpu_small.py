@@ -90,3 +90,37 @@ def test_all_check_shapes_in_one_launch(mld):
             outs.append(dec.decode(llr, syn, 9, want_post=True))
             torch.cuda.synchronize()
         _same(outs[0], outs[1])
+
+
+def test_concurrent_streams(mld):
+    """Decoders on their own threads and streams at the same time: each
+    cooperative launch gets its blocks together, whatever else runs."""
+    import threading
+    import torch
+    g0 = preset_graph(0.1, 16384, 3)
+    g = mld.Graph.from_edges(g0)
+    w = make_workload(0.1, 16384, 16, 3, 4300, beta=0.35, graph=g0)
+    y, sig, s = (torch.from_numpy(v).cuda() for v in (w.y, w.sigma, w.s))
+    ref = mld.Decoder(g, 16, msg_dtype="f16").decode_y(y, sig, s, 20, early_term=True, want_post=True)
+    torch.cuda.synchronize()
+    bad = []
+
+    def work():
+        try:
+            st = torch.cuda.Stream()
+            dec = mld.Decoder(g, 16, msg_dtype="f16")
+            with torch.cuda.stream(st):
+                for _ in range(40):
+                    out = dec.decode_y(y, sig, s, 20, early_term=True, want_post=True)
+                st.synchronize()
+                assert dec.status() == 0
+                _same(ref, out)
+        except BaseException as e:  # noqa: BLE001 -- reported by the main thread
+            bad.append(e)
+
+    threads = [threading.Thread(target=work) for _ in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
