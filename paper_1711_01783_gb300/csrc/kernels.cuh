@@ -506,13 +506,14 @@ struct TermsRing {
     }
 };
 
-// The update of one check, codewords lane0
-// .. lane0+3 of the slab; rout: its first message row there, e0 and s0 its
-// first core edge and degree-1 slot; valid false: compute but store nothing.  sb: the
-// check's syndrome bits for the 4 codewords (bit k: lane0 + k); donenib:
-// their converged flags under early termination.  The terms are read through t: lv(i) and ro(i), posterior and stored message of
-// core term i, p1(i), phi term of degree-1 term i.  LAY (layered schedule):
-// the check also owns its core VNs' posteriors and updates them in place.
+// The update of one check, codewords lane0 .. lane0+3 of the slab; rout: its
+// first message row there, e0 and s0 its first core edge and degree-1 slot;
+// valid false: compute but store nothing.  sb: the check's syndrome bits for
+// the 4 codewords (bit k: lane0 + k); donenib: their converged flags under
+// early termination.  The terms are read through t: lv(i) and ro(i), posterior
+// and stored message of core term i, p1(i), phi term of degree-1 term i.  LAY
+// (layered schedule): the check also owns its core VNs' posteriors and updates
+// them in place.
 template <typename MsgT, int W, int DC, int DD, int PASS, bool ACC, bool LAY, typename Terms>
 __device__ __forceinline__ void check_terms(const CnArgs &a, int lane0, int slab, bool valid, MsgT *rout,
                                                 int32_t e0, int32_t s0, uint32_t sb, uint32_t donenib, const Terms &t) {
@@ -1591,8 +1592,10 @@ constexpr int kVnLanes = 8;
 template <typename MsgT> struct VnRow;
 template <> struct VnRow<__half> {
     uint4 u;
+    template <bool ONCE>
     __device__ __forceinline__ void load(const __half *p, uint64_t policy) {
-        u = load_once(reinterpret_cast<const uint4 *>(p), policy);
+        if constexpr (ONCE) u = load_once(reinterpret_cast<const uint4 *>(p), policy);
+        else u = *reinterpret_cast<const uint4 *>(p);
     }
     __device__ __forceinline__ float2 pair(int i) const {
         const uint32_t w = i == 0 ? u.x : i == 1 ? u.y : i == 2 ? u.z : u.w;
@@ -1601,9 +1604,16 @@ template <> struct VnRow<__half> {
 };
 template <> struct VnRow<float> {
     float4 a, b;
+    template <bool ONCE>
     __device__ __forceinline__ void load(const float *p, uint64_t policy) {
-        a = load_once(reinterpret_cast<const float4 *>(p), policy);
-        b = load_once(reinterpret_cast<const float4 *>(p + 4), policy);
+        const float4 *q = reinterpret_cast<const float4 *>(p);
+        if constexpr (ONCE) {
+            a = load_once(q, policy);
+            b = load_once(q + 1, policy);
+        } else {
+            a = q[0];
+            b = q[1];
+        }
     }
     __device__ __forceinline__ float2 pair(int i) const {
         return i == 0 ? make_float2(a.x, a.y) : i == 1 ? make_float2(a.z, a.w) : i == 2 ? make_float2(b.x, b.y)
@@ -1616,7 +1626,9 @@ template <> struct VnRow<float> {
 // are formed in CSC order.  A message row is read once per pass: its lines go
 // past L1 and leave L2 first, so that they do not displace the posteriors,
 // which are stored to stay (the next check pass gathers each row once per
-// edge).  The pass is bound by HBM (each message row once, in the order of a
+// edge).  A row shorter than a line shares it with rows that are read later, so
+// it is loaded the ordinary way (8 codewords, n = 10^6, half, rows of 16 bytes:
+// 0.050 ms with evict-first, 0.042 ms without).  The pass is bound by HBM (each message row once, in the order of a
 // random permutation).  Rate 0.1, n = 10^6, 64 codewords, half, 4 codewords
 // per thread: 0.132 ms with plain loads and stores, 0.120 ms with the
 // priorities, and the check pass 0.285 -> 0.275 ms; 8 codewords per thread
@@ -1627,6 +1639,7 @@ template <typename MsgT, int W, int kRound = IsHalf<MsgT>::value ? 6 : 4>
 __device__ __forceinline__ void var_body(const VnArgs &a, int64_t t, int slab) {
     constexpr int TPV = W / kVnLanes;
     constexpr int NB = W / 8;
+    constexpr bool kOnce = W * sizeof(MsgT) >= 128;
     const int32_t v = static_cast<int32_t>(t / TPV);
     if (v >= a.n_core) return;
     const int lane0 = static_cast<int>(t % TPV) * kVnLanes;
@@ -1645,7 +1658,7 @@ __device__ __forceinline__ void var_body(const VnArgs &a, int64_t t, int slab) {
         for (int k = 0; k < kRound; ++k) e[k] = k < rem ? __ldg(a.vedge + j + k) : 0;
 #pragma unroll
         for (int k = 0; k < kRound; ++k)
-            if (k < rem) r[k].load(rb + static_cast<size_t>(e[k]) * W, once);
+            if (k < rem) r[k].template load<kOnce>(rb + static_cast<size_t>(e[k]) * W, once);
 #pragma unroll
         for (int k = 0; k < kRound; ++k) {
             if (k < rem) {
