@@ -1768,17 +1768,21 @@ __device__ __forceinline__ void syndrome_body(const SynArgs &a, int64_t first, i
     };
     // ORs the warp's failures into the slab's fail words, only bits not already
     // set (most warps of a failing slab then read the words instead of
-    // contending on them); returns the words
+    // contending on them); returns the words as the first lane read them, so
+    // that the whole warp decides alike (other warps change them meanwhile)
     uint32_t *fw = a.fail + slab * DW;
     auto publish = [&](unsigned long long x) {
         const uint32_t lo = __reduce_or_sync(0xFFFFFFFFu, static_cast<uint32_t>(x));
         const uint32_t hi = DW > 1 ? __reduce_or_sync(0xFFFFFFFFu, static_cast<uint32_t>(x >> 32)) : 0u;
-        const uint32_t f0 = *reinterpret_cast<volatile uint32_t *>(fw);
-        const uint32_t f1 = DW > 1 ? *reinterpret_cast<volatile uint32_t *>(fw + 1) : 0u;
+        uint32_t f0 = 0, f1 = 0;
         if ((threadIdx.x & 31) == 0) {
+            f0 = *reinterpret_cast<volatile uint32_t *>(fw);
+            if (DW > 1) f1 = *reinterpret_cast<volatile uint32_t *>(fw + 1);
             if (lo & ~f0) atomicOr(fw, lo);
             if (DW > 1 && (hi & ~f1)) atomicOr(fw + 1, hi);
         }
+        f0 = __shfl_sync(0xFFFFFFFFu, f0, 0);
+        if (DW > 1) f1 = __shfl_sync(0xFFFFFFFFu, f1, 0);
         return (lo | f0) | static_cast<unsigned long long>(hi | f1) << 32;
     };
     // once every codeword has failed a check (or is known), further checks

@@ -1,0 +1,62 @@
+"""The one-launch decode of small problems: graphs and batches at the edges of
+its phases, against the launch-per-phase path (the same call with the kernel
+timing hook on), exactly."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mld():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    import paper_1711_01783_gb300 as m
+    return m
+
+
+def _same(a, b):
+    for k in a:
+        if a[k] is not None:
+            assert np.array_equal(a[k].cpu().numpy(), b[k].cpu().numpy()), k
+
+
+def _decode(dec, llr, syn, iters, early, soft, timed):
+    import torch
+    dec.timing(1 if timed else 0)
+    out = dec.decode(llr, syn, iters, early_term=early, want_post=soft)
+    torch.cuda.synchronize()
+    assert dec.status() == 0
+    return out
+
+
+@pytest.mark.parametrize("msg,B", [("f16", 64), ("f16", 7), ("f32", 33)])
+def test_many_checks_a_thread_in_the_syndrome_phase(mld, msg, B):
+    """Eight checks with edges (rows and columns of a 4 x 3 array of VNs) and
+    3000 without: the decode runs in one block of 512 threads, whose warps
+    publish their first failures before they read the rest (more than four
+    checks a thread).  The edgeless checks of some codewords ask for a 1, so
+    those never converge."""
+    import torch
+    rng = np.random.default_rng(11)
+    nv, c = 12, 8
+    ev = np.array([[3 * j, 3 * j + 1, 3 * j + 2] for j in range(4)] + [[j, j + 4, j + 8] for j in range(4)],
+                  np.int32).reshape(-1)
+    ec = np.repeat(np.arange(c), 3).astype(np.int32)
+    m = c + 3000
+    g = mld.Graph(ev, ec, nv, m)
+    x = rng.integers(0, 2, (B, nv))
+    syn = np.zeros((B, m), np.uint8)
+    for j in range(c):
+        syn[:, j] = x[:, ev[3 * j:3 * j + 3]].sum(axis=1) & 1
+    syn[::3, c + 17::500] = 1
+    llr = ((1 - 2 * x) * 3.0 + rng.normal(0, 2, x.shape)).astype(np.float32)
+    llr_d, syn_d = torch.from_numpy(llr).cuda(), torch.from_numpy(syn).cuda()
+    dec = mld.Decoder(g, B, msg_dtype=msg)
+    for early in (True, False):
+        a = _decode(dec, llr_d, syn_d, 25, early, False, False)
+        b = _decode(dec, llr_d, syn_d, 25, early, False, True)
+        _same(a, b)
+        conv = a["converged"].cpu().numpy()
+        assert not conv[::3].any() and conv.any()
