@@ -9,6 +9,7 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "wrap_count.h"
 
 namespace {
 
@@ -48,8 +49,8 @@ struct SmallArgs {
 };
 
 // Grid barrier of a cooperative launch (every block is resident): arrivals are
-// counted up, and every block polls the count itself, one L2 round trip after
-// the last arrival.  Writes made before it are visible after it.  `target`:
+// counted up (modulo 2^32), and every block polls the count itself, one L2 round
+// trip after the last arrival.  Writes made before it are visible after it.  `target`:
 // the count of this barrier, raised for the next one.  A wait that runs out
 // (2 s) raises the abort flag and the block leaves (false); its decoder then
 // reports MLD_ETIMEOUT for good, and later launches leave at their first
@@ -65,7 +66,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t *bar, uint32_t &target) {
         unsigned long long t0 = 0;
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(bar) : "memory");
-            if (now >= target) break;
+            if (mld::count_reached(now, target)) break;
             if ((++spins & 1023u) == 0) {
                 uint32_t aborted;
                 asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(aborted) : "l"(bar + 2) : "memory");
