@@ -171,7 +171,12 @@ __global__ void __launch_bounds__(kSmallBlock, 1) k_small_decode(SmallArgs s) {
     cn.done = vn.done = sy.done = done;
     const uint32_t step = gridDim.x * blockDim.x;
     const uint32_t t0 = ((threadIdx.x / 32) * gridDim.x + blockIdx.x) * 32 + threadIdx.x % 32;
+    // the variables of every slab are one range of threads; each slab's checks go
+    // to a share of the warps (to all of them if it is the only slab)
     const uint32_t vn_threads = static_cast<uint32_t>(vn.n_core) * (W / kVnLanes);
+    const uint32_t vn_total = vn_threads * s.slabs;
+    const int warps = static_cast<int>(step / 32), groups = min(s.slabs, warps), per = warps / groups;
+    const int warp = static_cast<int>(t0 / 32);
     uint32_t target = 0;
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < 2 * words; i += blockDim.x) s.fail[i] = 0u;
@@ -184,9 +189,10 @@ __global__ void __launch_bounds__(kSmallBlock, 1) k_small_decode(SmallArgs s) {
         else small_checks<MsgT, W, kPassFull>(s, cn, t0, step);
         if (!grid_barrier(s.bar, target)) break;
         vn.want_bits = cn.final_pass;
-        for (int slab = 0; slab < s.slabs; ++slab) {
+        for (uint32_t t = t0; t < vn_total; t += step) {
+            const uint32_t slab = s.slabs == 1 ? 0u : t / vn_threads;
             if (et && slab_all_done<W>(done, slab)) continue;
-            for (uint32_t t = t0; t < vn_threads; t += step) var_body<MsgT, W, kSmallRound<MsgT>>(vn, t, slab);
+            var_body<MsgT, W, kSmallRound<MsgT>>(vn, t - slab * vn_threads, slab);
         }
         // the fail words of the other parity: every block has read them
         if (blockIdx.x == 0)
@@ -196,9 +202,9 @@ __global__ void __launch_bounds__(kSmallBlock, 1) k_small_decode(SmallArgs s) {
         uint32_t *f = s.fail + (l & 1) * words;
         sy.fail = f;
         sy.hb1 = cn.hb1;
-        for (int slab = 0; slab < s.slabs; ++slab) {
+        for (int slab = warp / per; slab < s.slabs && warp < groups * per; slab += groups) {
             if (et && slab_all_done<W>(done, slab)) continue;
-            syndrome_body<W>(sy, t0, step, slab);
+            syndrome_body<W>(sy, (warp % per) * 32 + threadIdx.x % 32, per * 32, slab);
         }
         if (!grid_barrier(s.bar, target)) break;
         // every block forms the same lane state from the same words

@@ -60,3 +60,29 @@ def test_many_checks_a_thread_in_the_syndrome_phase(mld, msg, B):
         _same(a, b)
         conv = a["converged"].cpu().numpy()
         assert not conv[::3].any() and conv.any()
+
+
+def _grid_graph(mld, rows, cols):
+    """VNs in an array, a check per row and per column (every VN of degree 2)."""
+    vn = np.arange(rows * cols, dtype=np.int32).reshape(rows, cols)
+    ev = np.concatenate([vn.reshape(-1), vn.T.reshape(-1)])
+    ec = np.concatenate([np.repeat(np.arange(rows), cols), rows + np.repeat(np.arange(cols), rows)]).astype(np.int32)
+    return mld.Graph(ev, ec, rows * cols, rows + cols)
+
+
+# 4 checks: one block of 16 warps with 17, 16 and 3 slabs of 8 (more slabs than
+# warps, as many, and a share that leaves a warp over); the same with the most
+# codewords of the path; 12 checks and 5 slabs of 32
+@pytest.mark.parametrize("side,B,W,msg", [(2, 135, 8, "f16"), (2, 128, 8, "f32"), (2, 20, 8, "f16"),
+                                          (2, 512, 64, "f16"), (6, 130, 32, "f32")])
+@pytest.mark.parametrize("early", [False, True])
+def test_batches_of_several_slabs(mld, side, B, W, msg, early):
+    """The slabs' variables and checks are spread over all warps."""
+    import torch
+    rng = np.random.default_rng(side + B)
+    g = _grid_graph(mld, side, side)
+    llr = torch.from_numpy(rng.normal(0.5, 1.5, (B, g.n_vn)).astype(np.float32)).cuda()
+    syn = torch.zeros((B, g.n_cn), dtype=torch.uint8, device="cuda")
+    syn[::5, 0] = 1
+    dec = mld.Decoder(g, B, msg_dtype=msg, slab_width=W)
+    _same(_decode(dec, llr, syn, 11, early, True, False), _decode(dec, llr, syn, 11, early, True, True))
