@@ -25,6 +25,18 @@ constexpr int kSmallMaxLanes = 512;    // codewords (their bookkeeping is in sha
 // codewords, half (944 000) 2.04 / 1.95 ms; n = 131072, 64 codewords 4.17 /
 // 3.44 ms.
 constexpr int64_t kSmallMaxThreads = 152 * 512 * 8;
+// A block takes a whole SM's registers, so a decode excludes other one-launch
+// decodes from its SMs until it ends.  One whose check threads all fit half of
+// the SMs takes no more than these: two such decodes run side by side.
+// Microseconds a decode of 25 iterations (n = 4096, half, early termination) on
+// 1 / 2 / 4 streams at once, 16 codewords: 390 / 753 / 1481 on as many SMs as
+// its warps spread over, 393 / 416 / 788 on half of them; 32 codewords (29 000
+// threads) 399 / 770 / 1516 and 408 / 423 / 811.  A larger decode keeps every
+// SM: on half of them a single one of 64 codewords (59 000 threads) takes 440
+// instead of 405, of 118 000 threads 538 instead of 446.  Several of those on
+// streams of their own take turns (64 codewords: 405 / 766 / 1503; with a launch
+// per phase 587 / 651 / 735); one batch or a plan serves them better.
+constexpr int kSmallShareDiv = 2;
 // edges in flight per thread in the variable update: the phase has few warps,
 // so a VN's rows are requested in two or three rounds
 template <typename MsgT> constexpr int kSmallRound = IsHalf<MsgT>::value ? 12 : 6;
@@ -285,8 +297,10 @@ bool launch_small(mld_decoder *d, int32_t batch, int32_t iters, bool et, bool ha
     }
     s.first[s.n_cls] = static_cast<uint32_t>(at);
     if (static_cast<uint64_t>(s.vn.n_core) * (W / kVnLanes) > static_cast<uint64_t>(kSmallMaxThreads)) return false;
-    // at least four warps a block, one block per SM at most
-    const int blocks = static_cast<int>(std::max<uint64_t>(1, std::min<uint64_t>(sm_count, (at + 127) / 128)));
+    // at least four warps a block, one block per SM at most (kSmallShareDiv)
+    const int part = std::max(1, sm_count / kSmallShareDiv);
+    const bool fits = at <= static_cast<uint64_t>(part) * kSmallBlock;
+    const int blocks = static_cast<int>(std::max<uint64_t>(1, std::min<uint64_t>(fits ? part : sm_count, (at + 127) / 128)));
     void *args[] = {&s};
     if (cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(&k_small_decode<MsgT, W>), dim3(blocks),
                                     dim3(kSmallBlock), args, 0, st) != cudaSuccess) {
