@@ -326,8 +326,10 @@ int mld_decoder_destroy(mld_decoder *d);
  * Flooding sum-product gather decodes of small problems (up to ~600 000
  * threads of a check update, checks of one to six core edges and at most one
  * degree-1 VN) run their iterations in one cooperative launch whose blocks
- * wait on one another at most 2 s; should such a wait run out, the results are
- * invalid and mld_decode_status returns MLD_ETIMEOUT from then on. */
+ * wait on one another at most 2 s.  Should such a wait run out, the decode
+ * gives up: converged and iters_used are 0 for every codeword, bits and
+ * posteriors are unfinished, and mld_decode_status returns MLD_ETIMEOUT from
+ * then on (later decodes of this kind on that decoder give up at once). */
 int mld_decode(mld_decoder *d, const float *llr, const uint8_t *syndrome,
                int32_t batch, int32_t max_iters, uint32_t flags,
                uint8_t *bits_out, float *post_out, uint8_t *converged,
@@ -354,13 +356,14 @@ int mld_decode_y(mld_decoder *d, const float *y, const float *sigma,
  * status word with a blocking copy; call after the stream is idle. */
 int mld_decode_status(mld_decoder *d);
 
-/* Test of the timeout path of the staged check update: with bytes > 0, every
- * later staged check-update launch of this decoder makes one block expect
- * `bytes` more than its first stage's copies bring, so that block's bounded
- * wait (2 s) runs out, it records MLD_ETIMEOUT in the status word and leaves
- * without storing (the decode's results are then invalid); 0 turns it off.
- * No fault is raised and the context stays usable.  Decoders without staging
- * ignore it.  A change waits for the device to be idle (it drops the
+/* Test of the bounded waits: with bytes > 0, every later staged check-update
+ * launch of this decoder makes one block expect `bytes` more than its first
+ * stage's copies bring, so that block's bounded wait (2 s) runs out, it records
+ * MLD_ETIMEOUT in the status word and leaves without storing (the decode's
+ * results are then invalid), and every later one-launch decode waits at its
+ * first barrier for an arrival that never comes and gives up (see mld_decode);
+ * 0 turns it off.  No fault is raised and the context stays usable.  Other
+ * decodes ignore it.  A change waits for the device to be idle (it drops the
  * decoder's captured early-termination loops).  Errors: MLD_EINVAL (null
  * decoder, bytes outside [0, 65536]), MLD_ECUDA. */
 int mld_decoder_test_stall(mld_decoder *d, int32_t bytes);
@@ -524,6 +527,10 @@ int mld_decoder_timing_read(mld_decoder *d, mld_timing *out);
  * call's contents; each call clears what must start at zero.  Calls whose
  * work overlaps on the GPU (different streams, or host threads racing)
  * corrupt each other: serialize them.
+ * A small problem's one launch (see mld_decode) may give up after 2 s; there is
+ * no decoder to ask for a status, so its sign is iters_used = 0 (with
+ * converged = 0) for every codeword of a call with max_iters > 0.  The next
+ * call starts afresh.
  * Errors: MLD_EINVAL (null pointer, bad dtype/flag/size, scratch too small),
  * MLD_ECUDA. */
 #define MLD_NOALLOC_SCRATCH_BYTES (32u * 1024u * 1024u)

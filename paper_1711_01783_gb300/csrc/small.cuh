@@ -57,16 +57,16 @@ struct SmallArgs {
     int32_t *iters_out;   // the caller's arrays, or null
     uint8_t *conv_out;
     uint32_t *bar;        // grid barrier: arrivals, generation, abort flag
-    int32_t *status;
+    int32_t *status;      // may be null
+    int32_t stall;        // test of the timeout path: arrivals that never come
 };
 
 // Grid barrier of a cooperative launch (every block is resident): arrivals are
 // counted up (modulo 2^32), and every block polls the count itself, one L2 round
 // trip after the last arrival.  Writes made before it are visible after it.  `target`:
 // the count of this barrier, raised for the next one.  A wait that runs out
-// (2 s) raises the abort flag and the block leaves (false); its decoder then
-// reports MLD_ETIMEOUT for good, and later launches leave at their first
-// barrier.
+// (2 s) raises the abort flag, on which every block leaves (false); the flag
+// stays up, and later launches with the same barrier words leave on entry.
 __device__ __forceinline__ bool grid_barrier(uint32_t *bar, uint32_t &target) {
     target += gridDim.x;
     int ok = 1;
@@ -95,8 +95,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t *bar, uint32_t &target) {
     return __syncthreads_and(ok) != 0;
 }
 
-// The last block to leave resets the barrier for the next launch (after a
-// timeout nothing is reset: the abort flag stays up).
+// The last block to leave resets the barrier for the next launch.
 __device__ __forceinline__ void grid_leave(uint32_t *bar) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -189,17 +188,20 @@ __global__ void __launch_bounds__(kSmallBlock, 1) k_small_decode(SmallArgs s) {
     const uint32_t vn_total = vn_threads * s.slabs;
     const int warps = static_cast<int>(step / 32), groups = min(s.slabs, warps), per = warps / groups;
     const int warp = static_cast<int>(t0 / 32);
-    uint32_t target = 0;
+    uint32_t target = s.stall > 0 ? 1u : 0u;
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < 2 * words; i += blockDim.x) s.fail[i] = 0u;
-    __syncthreads();
-    for (int32_t l = 1; l <= s.iters; ++l) {
+    uint32_t aborted = 0;
+    if (threadIdx.x == 0)
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(aborted) : "l"(s.bar + 2) : "memory");
+    bool up = __syncthreads_or(static_cast<int>(aborted)) == 0;  // no wait has run out
+    for (int32_t l = 1; up && l <= s.iters; ++l) {
         const bool last = l == s.iters;
         cn.final_pass = (last || et) ? 1 : 0;
         cn.hb1 = s.cn.hb1 + (l & 1) * s.h1;
         if (s.hard1) small_checks<MsgT, W, kPassHard>(s, cn, t0, step);
         else small_checks<MsgT, W, kPassFull>(s, cn, t0, step);
-        if (!grid_barrier(s.bar, target)) break;
+        if (!(up = grid_barrier(s.bar, target))) break;
         vn.want_bits = cn.final_pass;
         for (uint32_t t = t0; t < vn_total; t += step) {
             const uint32_t slab = s.slabs == 1 ? 0u : t / vn_threads;
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(kSmallBlock, 1) k_small_decode(SmallArgs s) {
         // the fail words of the other parity: every block has read them
         if (blockIdx.x == 0)
             for (int i = threadIdx.x; i < words; i += blockDim.x) s.fail[(1 - (l & 1)) * words + i] = 0u;
-        if (!grid_barrier(s.bar, target)) break;
+        if (!(up = grid_barrier(s.bar, target))) break;
         if (!cn.final_pass) continue;
         uint32_t *f = s.fail + (l & 1) * words;
         sy.fail = f;
@@ -218,7 +220,7 @@ __global__ void __launch_bounds__(kSmallBlock, 1) k_small_decode(SmallArgs s) {
             if (et && slab_all_done<W>(done, slab)) continue;
             syndrome_body<W>(sy, (warp % per) * 32 + threadIdx.x % 32, per * 32, slab);
         }
-        if (!grid_barrier(s.bar, target)) break;
+        if (!(up = grid_barrier(s.bar, target))) break;
         // every block forms the same lane state from the same words
         for (int i = threadIdx.x; i < words; i += blockDim.x) fail[i] = __ldcg(f + i);
         __syncthreads();
@@ -238,21 +240,20 @@ __global__ void __launch_bounds__(kSmallBlock, 1) k_small_decode(SmallArgs s) {
             if (all) break;
         }
     }
+    // given up: no codeword counts as converged, after 0 iterations, and the
+    // barrier is not reset
     if (blockIdx.x == 0) {
-        uint32_t aborted;
-        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(aborted) : "l"(s.bar + 2) : "memory");
-        if (aborted) {
-            if (threadIdx.x == 0 && s.status) atomicCAS(s.status, 0, MLD_ETIMEOUT);
-            return;
-        }
+        if (!up && threadIdx.x == 0 && s.status) atomicCAS(s.status, 0, MLD_ETIMEOUT);
         for (int b = threadIdx.x; b < s.batch; b += blockDim.x) {
-            s.iters_dev[b] = its[b];
-            s.conv_dev[b] = conv[b];
-            if (s.iters_out) s.iters_out[b] = its[b];
-            if (s.conv_out) s.conv_out[b] = conv[b];
+            const int32_t it = up ? its[b] : 0;
+            const uint8_t cv = up ? conv[b] : 0;
+            s.iters_dev[b] = it;
+            s.conv_dev[b] = cv;
+            if (s.iters_out) s.iters_out[b] = it;
+            if (s.conv_out) s.conv_out[b] = cv;
         }
     }
-    grid_leave(s.bar);
+    if (up) grid_leave(s.bar);
 }
 
 // Runs the iterations in one launch on st; false if the problem is not small or
@@ -278,6 +279,7 @@ bool launch_small(mld_decoder *d, int32_t batch, int32_t iters, bool et, bool ha
     s.conv_out = conv_out;
     s.bar = d->bar;
     s.status = d->status;
+    s.stall = d->stall_test;
     s.cn = CnArgs{g->cptr, g->col, g->dptr, h.n_cn, h.n_core, h.n_deg1, h.e_core, d->r, d->Lv, d->lch1, d->phi1,
                   d->post1, d->hb1, d->sbits, nullptr, d->lmax_i, d->amin_i, 0, et ? 1 : 0};
     if (!et && !soft) s.cn.post1 = nullptr;

@@ -86,3 +86,49 @@ def test_batches_of_several_slabs(mld, side, B, W, msg, early):
     syn[::5, 0] = 1
     dec = mld.Decoder(g, B, msg_dtype=msg, slab_width=W)
     _same(_decode(dec, llr, syn, 11, early, True, False), _decode(dec, llr, syn, 11, early, True, True))
+
+
+@pytest.mark.parametrize("early", [False, True])
+def test_a_wait_that_runs_out_is_reported(mld, early):
+    """A decode whose first barrier waits for an arrival that never comes
+    (mld_decoder_test_stall) gives up after 2 s: no codeword counts as
+    converged, whatever the output arrays held, in device and in host memory;
+    the status says so, and later decodes of that decoder give up at once.  A
+    new decoder is clean."""
+    import time
+    import torch
+    from synthetic import make_workload
+    w = make_workload(0.1, 4096, 8, 3, 4400, beta=0.3)
+    g = mld.Graph.from_edges(w.graph)
+    y, sig, s = (torch.from_numpy(v).cuda() for v in (w.y, w.sigma, w.s))
+    dec = mld.Decoder(g, 8, msg_dtype="f16")
+    ref = dec.decode_y(y, sig, s, 30, early_term=early)
+    torch.cuda.synchronize()
+    assert dec.status() == 0 and ref["converged"].all()
+
+    def call(host):
+        n = g.n_vn
+        out = dict(bits=torch.zeros((8, n), dtype=torch.uint8), post=None,
+                   converged=torch.full((8,), 1, dtype=torch.uint8), iters_used=torch.full((8,), 9, dtype=torch.int32))
+        out = {k: v if v is None else (v.numpy() if host else v.cuda()) for k, v in out.items()}
+        t0 = time.time()
+        if host:
+            dec.decode_y(w.y, w.sigma, w.s, 30, early_term=early, out=out)
+        else:
+            dec.decode_y(y, sig, s, 30, early_term=early, out=out)
+        torch.cuda.synchronize()
+        assert dec.status() == mld.MLD_ETIMEOUT
+        for k in ("converged", "iters_used"):
+            assert not np.asarray(out[k] if host else out[k].cpu()).any(), k
+        return time.time() - t0
+
+    dec.test_stall(1)
+    dt = call(False)
+    assert 1.9 < dt < 60, dt
+    dec.test_stall(0)
+    assert call(False) < 1.5 and call(True) < 1.5
+    fresh = mld.Decoder(g, 8, msg_dtype="f16")
+    got = fresh.decode_y(y, sig, s, 30, early_term=early)
+    torch.cuda.synchronize()
+    assert fresh.status() == 0
+    _same(ref, got)
