@@ -356,6 +356,10 @@ int mld_decode_y(mld_decoder *d, const float *y, const float *sigma,
  * status word with a blocking copy; call after the stream is idle. */
 int mld_decode_status(mld_decoder *d);
 
+/* Number of this decoder's decode calls so far whose iterations were enqueued
+ * as one cooperative launch (see mld_decode).  Errors: MLD_EINVAL. */
+int mld_decoder_one_launch(const mld_decoder *d, int64_t *decodes);
+
 /* Test of the bounded waits: with bytes > 0, every later staged check-update
  * launch of this decoder makes one block expect `bytes` more than its first
  * stage's copies bring, so that block's bounded wait (2 s) runs out, it records

@@ -59,6 +59,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
         uint8_t *co = out_dev ? conv_out : nullptr;
         if constexpr (IsHalf<MsgT>::value) small = mld::small_decode_f16(d, W, batch, iters, et, hard, io, co, sm_count, st, post != nullptr);
         else small = mld::small_decode_f32(d, W, batch, iters, et, hard, io, co, sm_count, st, post != nullptr);
+        d->one_launch += small ? 1 : 0;
     }
     if (!small) MLD_CUDA(cudaMemsetAsync(d->done, 0, sizeof(uint32_t) * slabs * DW, st));
 

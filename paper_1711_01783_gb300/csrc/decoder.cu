@@ -510,6 +510,13 @@ int mld_decode_status(mld_decoder *d) {
     return v[0] == 0 ? MLD_OK : mld::fail(v[0], graph_fault_text(v));
 }
 
+int mld_decoder_one_launch(const mld_decoder *d, int64_t *decodes) {
+    mld::clear_error();
+    if (!d || !decodes) return mld::fail(MLD_EINVAL, "decoder_one_launch: null pointer");
+    *decodes = d->one_launch;
+    return MLD_OK;
+}
+
 int mld_decoder_test_stall(mld_decoder *d, int32_t bytes) {
     mld::clear_error();
     if (!d) return mld::fail(MLD_EINVAL, "decoder_test_stall: null decoder");

@@ -2247,6 +2247,7 @@ struct mld_decoder {
     cudaStream_t cap = nullptr;
     int32_t *lctr = nullptr;
     uint32_t *bar = nullptr;  // grid barrier of the one-launch decode (3 words, zero between launches)
+    int64_t one_launch = 0;   // decodes enqueued that way
     struct LoopGraph { int32_t batch, variant; uint64_t layers_gen; cudaGraphExec_t exec; };
     std::vector<LoopGraph> loops;
     float *Lv2 = nullptr, *Lv3 = nullptr;

@@ -25,9 +25,11 @@ def _same(a, b):
 def _decode(dec, llr, syn, iters, early, soft, timed):
     import torch
     dec.timing(1 if timed else 0)
+    before = dec.one_launch_decodes()
     out = dec.decode(llr, syn, iters, early_term=early, want_post=soft)
     torch.cuda.synchronize()
     assert dec.status() == 0
+    assert dec.one_launch_decodes() - before == (0 if timed else 1)
     return out
 
 
@@ -132,3 +134,66 @@ def test_a_wait_that_runs_out_is_reported(mld, early):
     torch.cuda.synchronize()
     assert fresh.status() == 0
     _same(ref, got)
+
+
+@pytest.mark.parametrize("msg", ["f32", "f16"])
+@pytest.mark.parametrize("early,soft", [(False, False), (False, True), (True, False), (True, True)])
+def test_every_check_shape_in_every_pass(mld, msg, early, soft):
+    """Checks of one to six core edges, with and without a degree-1 VN: fixed
+    iterations, the decisions-only pass and the soft early-terminated one.
+    The channel values are strong enough for some codewords to stop early."""
+    import torch
+    rng = np.random.default_rng(6)
+    nv, ev, ec, c = 160, [], [], 0
+    order = np.concatenate([rng.permutation(160) for _ in range(4)]).tolist()
+    for _ in range(10):
+        for dc in range(1, 7):
+            for dd in (0, 1):
+                row = []
+                while len(row) < dc:
+                    v = order.pop(0)
+                    (order if v in row else row).append(v)
+                ev += row + ([nv] if dd else [])
+                ec += [c] * (dc + dd)
+                nv += dd
+                c += 1
+    g = mld.Graph(np.array(ev, np.int32), np.array(ec, np.int32), nv, c)
+    B = 21
+    x = rng.integers(0, 2, (B, nv)).astype(np.uint8)
+    syn = np.zeros((B, c), np.uint8)
+    for v, k in zip(ev, ec):
+        syn[:, k] ^= x[:, v]
+    scale = np.where(np.arange(B) % 2, 1.0, 4.0)[:, None]
+    llr = (scale * (1 - 2.0 * x) + rng.normal(0, 1.2, x.shape)).astype(np.float32)
+    llr, syn = torch.from_numpy(llr).cuda(), torch.from_numpy(syn).cuda()
+    dec = mld.Decoder(g, B, msg_dtype=msg)
+    one = _decode(dec, llr, syn, 12, early, soft, False)
+    _same(one, _decode(dec, llr, syn, 12, early, soft, True))
+    its = one["iters_used"].cpu().numpy()
+    assert (its.min() < its.max()) if early else (its == 12).all()
+
+
+@pytest.mark.parametrize("rate,n,B,msg,W,small", [
+    (0.1, 4096, 1, "f32", 0, True), (0.05, 5001, 33, "f32", 0, True), (0.02, 5001, 65, "f16", 0, True),
+    (0.1, 4096, 16, "f16", 64, True), (0.05, 3000, 140, "f32", 0, True),
+    (0.1, 16384, 16, "f16", 0, True),     # a class of six core edges and a degree-1 VN
+    (0.1, 65536, 64, "f16", 0, False),    # past the size limit
+])
+def test_which_decodes_run_in_one_launch(mld, rate, n, B, msg, W, small):
+    import torch
+    from synthetic import make_workload
+    w = make_workload(rate, n, B, 3, 4200 + B, beta=0.35)
+    g = mld.Graph.from_edges(w.graph)
+    dec = mld.Decoder(g, B, msg_dtype=msg, slab_width=W)
+    dec.decode_y(*(torch.from_numpy(v).cuda() for v in (w.y, w.sigma, w.s)), 3)
+    torch.cuda.synchronize()
+    assert dec.one_launch_decodes() == (1 if small else 0)
+
+
+def test_checks_of_seven_core_edges_keep_a_launch_per_phase(mld):
+    import torch
+    g = _grid_graph(mld, 7, 7)
+    dec = mld.Decoder(g, 4)
+    dec.decode(torch.ones((4, 49), device="cuda"), torch.zeros((4, 14), dtype=torch.uint8, device="cuda"), 3)
+    torch.cuda.synchronize()
+    assert dec.one_launch_decodes() == 0 and dec.status() == 0
