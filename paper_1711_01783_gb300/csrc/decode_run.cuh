@@ -69,7 +69,8 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
     auto hb1_of = [&](int32_t l) { return d->hb1 + static_cast<size_t>(l & 1) * h1; };
     CnArgs ca{g->cptr, g->col, g->dptr, h.n_cn, h.n_core, h.n_deg1, h.e_core,
               d->r, d->Lv, d->lch1, d->phi1, d->post1, d->hb1, d->sbits, d->done,
-              d->lmax_i, d->amin_i, 0, et ? 1 : 0, batch};
+              d->lmax_i, d->amin_i, 0, et ? 1 : 0};
+    ca.batch = batch;
     ca.status = d->status;
     ca.stall_test = d->stall_test;
     if (!et && !post) ca.post1 = nullptr;  // nothing reads the degree-1 posteriors
@@ -78,7 +79,7 @@ int run_decode(mld_decoder *d, const float *in, const float *sigma, const uint8_
     // early termination without soft output: degree-1 decisions only (a
     // sum-product property)
     const bool hard1 = et && !post && d->check_rule == MLD_CHECK_SUM_PRODUCT;
-    VnArgs va{g->vptr, g->vedge, h.n_core, h.e_core, d->r, d->lch, d->Lv, d->hb_core, d->done, 0, et ? 1 : 0, batch};
+    VnArgs va{g->vptr, g->vedge, h.n_core, h.e_core, d->r, d->lch, d->Lv, d->hb_core, d->done, 0, et ? 1 : 0};
     SynArgs sa{g->cptr, g->col, g->dptr, h.n_cn, h.n_core, h.n_deg1, d->sbits, d->hb_core, d->hb1,
                d->fail, d->done, et ? 1 : 0, batch};
     // check-update launches, one per check class (built with the graph)

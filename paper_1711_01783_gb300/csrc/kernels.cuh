@@ -310,22 +310,23 @@ __device__ __forceinline__ unsigned pair_mask() {
     return 0x3u << ((threadIdx.x & 31u) & ~1u);
 }
 
-// Which of the N codewords from lane0 of a slab have stopped (a.done), as the
-// bits of the threads that keep their values.  Lanes past the batch count as
-// stopped in a.done but are left out here: nothing reads them, and a thread
-// that owns only such lanes would reload every row to write it back (33
-// codewords of n = 200000 in a slab of 64, rate 0.02, half, soft output: 129 us
-// an iteration, 101 us without; storing nothing for them leaves part-written
-// lines, 143 us).
-template <int W, int N, typename Args>
-__device__ __forceinline__ uint32_t stopped_lanes(const Args &a, int slab, int lane0) {
+// done-bit nibble of the 4 codewords starting at lane0 of a slab
+template <int W>
+__device__ __forceinline__ uint32_t done_nibble(const uint32_t *done, int slab, int lane0) {
     constexpr int DW = (W + 31) / 32;
-    const int real = min(max(a.batch - slab * W - lane0, 0), N);
-    return (a.done[slab * DW + lane0 / 32] >> (lane0 & 31)) & ((1u << real) - 1u);
+    return (done[slab * DW + lane0 / 32] >> (lane0 & 31)) & 0xFu;
 }
-template <int W, typename Args>
-__device__ __forceinline__ uint32_t stopped_nibble(const Args &a, int slab, int lane0) {
-    return stopped_lanes<W, 4>(a, slab, lane0);
+
+// Those whose values a check pass keeps.  Lanes past the batch count as done
+// but are left out where messages and degree-1 posteriors would be reloaded to
+// be written back (MASK): nothing reads them (33 codewords of n = 200000 in a
+// slab of 64 of a plan, rate 0.02, half, soft output: 129 us an iteration, 101 us
+// without; storing nothing for them leaves part-written lines, 143 us).
+template <int W, bool MASK, typename Args>
+__device__ __forceinline__ uint32_t kept_nibble(const Args &a, int slab, int lane0) {
+    const uint32_t d = done_nibble<W>(a.done, slab, lane0);
+    if constexpr (!MASK) return d;
+    return d & ((1u << min(max(a.batch - slab * W - lane0, 0), 4)) - 1u);
 }
 
 template <int W>
@@ -353,7 +354,6 @@ struct CnArgs {
     const uint32_t *done;  // [slab][ceil(W/32)] converged lanes (ET)
     float lmax, amin;
     int final_pass, et;
-    int32_t batch;
     // Posterior accumulation (fixed iterations only): each new message, as
     // stored, is added to this [slab][n_core][W] array, which holds L_ch on
     // entry and L_v of this iteration (Eq. 4) once the pass is complete.
@@ -370,6 +370,7 @@ struct CnArgs {
     // (0, 0) of a staged check update expects for its first stage, so that
     // its wait runs out (0: none).
     int32_t stall_test;
+    int32_t batch;  // codewords (read with et)
 };
 
 enum { kRuleSumProduct = 0, kRuleMinSum = 1 };
@@ -692,7 +693,7 @@ __device__ __forceinline__ void check_irregular(const CnArgs &a, const ClassLaun
     const uint32_t sb =
         (static_cast<uint32_t>(a.sbits[(static_cast<size_t>(slab) * a.n_cn + c) * NB + lane0 / 8]) >>
          (lane0 & 7));
-    const uint32_t donenib = a.et ? stopped_nibble<W>(a, slab, lane0) : 0u;
+    const uint32_t donenib = a.et ? kept_nibble<W, true>(a, slab, lane0) : 0u;
     MsgT *rb = static_cast<MsgT *>(a.r) + static_cast<size_t>(slab) * a.e_core * W + lane0;
     const float *lvb = a.Lv + static_cast<size_t>(slab) * a.n_core * W + lane0;
     const float *l1b = a.lch1 + static_cast<size_t>(slab) * a.n_deg1 * W + lane0;
@@ -779,7 +780,7 @@ __device__ __forceinline__ void check_class_body(const CnArgs &a, const ClassLau
     const float *lvb = a.Lv + static_cast<size_t>(slab) * a.n_core * W + lane0;
     const float *pb = a.phi1 + (static_cast<size_t>(slab) * a.n_deg1 + cl.s0) * W + lane0;
     const uint8_t *sbp = a.sbits + (static_cast<size_t>(slab) * a.n_cn + cl.c0) * NB + lane0 / 8;
-    const uint32_t donenib = (PASS != kPassPlain && a.et) ? stopped_nibble<W>(a, slab, lane0) : 0u;
+    const uint32_t donenib = (PASS != kPassPlain && a.et) ? kept_nibble<W, PASS == kPassFull>(a, slab, lane0) : 0u;
     const int32_t stride = blocks * (kBlock / TPC);
     const uint32_t sm = smem_u32(smem);
     int32_t v[DC > 0 ? DC : 1];  // column indices of the check whose operands are requested next,
@@ -1031,7 +1032,7 @@ __global__ void __launch_bounds__(kBlock, kStagedBlocksPerSm) k_check_staged(CnA
     if (s < stages) issue(s, 0, vn);
     cols_of(s + step, vn);
     uint32_t sbn = s < stages ? sb_of(s) : 0u;
-    const uint32_t donenib = a.et ? stopped_nibble<W>(a, slab, lane0) : 0u;
+    const uint32_t donenib = a.et ? done_nibble<W>(a.done, slab, lane0) : 0u;
     for (int k = 0; s < stages; s += step, ++k) {
         const int buf = k & 1;
         const int32_t sn = s + step;
@@ -1264,7 +1265,7 @@ __device__ __forceinline__ void check_layered_irregular(const CnArgs &a, int32_t
     const uint32_t sb =
         (static_cast<uint32_t>(a.sbits[(static_cast<size_t>(slab) * a.n_cn + c) * NB + lane0 / 8]) >>
          (lane0 & 7));
-    const uint32_t donenib = a.et ? stopped_nibble<W>(a, slab, lane0) : 0u;
+    const uint32_t donenib = a.et ? done_nibble<W>(a.done, slab, lane0) : 0u;
     MsgT *rb = static_cast<MsgT *>(a.r) + static_cast<size_t>(slab) * a.e_core * W + lane0;
     float *lvb = const_cast<float *>(a.Lv) + static_cast<size_t>(slab) * a.n_core * W + lane0;
     const float *l1b = a.lch1 + static_cast<size_t>(slab) * a.n_deg1 * W + lane0;
@@ -1404,7 +1405,7 @@ __device__ __forceinline__ void check_minsum(const CnArgs &a, const ClassLaunch 
     const uint32_t sb =
         (static_cast<uint32_t>(a.sbits[(static_cast<size_t>(slab) * a.n_cn + c) * NB + lane0 / 8]) >>
          (lane0 & 7));
-    const uint32_t donenib = a.et ? stopped_nibble<W>(a, slab, lane0) : 0u;
+    const uint32_t donenib = a.et ? done_nibble<W>(a.done, slab, lane0) : 0u;
     MsgT *rb = static_cast<MsgT *>(a.r) + static_cast<size_t>(slab) * a.e_core * W + lane0;
     const float *lvb = a.Lv + static_cast<size_t>(slab) * a.n_core * W + lane0;
     const float *l1b = a.lch1 + static_cast<size_t>(slab) * a.n_deg1 * W + lane0;
@@ -1474,7 +1475,7 @@ __device__ __forceinline__ void check_minsum_irregular(const CnArgs &a, int32_t 
     const uint32_t sb =
         (static_cast<uint32_t>(a.sbits[(static_cast<size_t>(slab) * a.n_cn + c) * NB + lane0 / 8]) >>
          (lane0 & 7));
-    const uint32_t donenib = a.et ? stopped_nibble<W>(a, slab, lane0) : 0u;
+    const uint32_t donenib = a.et ? done_nibble<W>(a.done, slab, lane0) : 0u;
     MsgT *rb = static_cast<MsgT *>(a.r) + static_cast<size_t>(slab) * a.e_core * W + lane0;
     const float *lvb = a.Lv + static_cast<size_t>(slab) * a.n_core * W + lane0;
     const float *l1b = a.lch1 + static_cast<size_t>(slab) * a.n_deg1 * W + lane0;
@@ -1596,7 +1597,6 @@ struct VnArgs {
     uint8_t *hb;        // [slab][n_core][W/8]
     const uint32_t *done;
     int want_bits, et;
-    int32_t batch;  // (read with et)
 };
 
 // One thread owns 8 codewords of one VN: 16 bytes of a half row (one load), 32
@@ -1684,7 +1684,8 @@ __device__ __forceinline__ void var_body(const VnArgs &a, int64_t t, int slab) {
     float *lv = a.Lv + vrow;
     if (a.et) {
         // converged lanes keep the posterior of their last iteration
-        const uint32_t dn = stopped_lanes<W, kVnLanes>(a, slab, lane0);
+        constexpr int DW = (W + 31) / 32;
+        const uint32_t dn = (a.done[slab * DW + lane0 / 32] >> (lane0 & 31)) & 0xFFu;
         if (dn) {
             const float4 p0 = *reinterpret_cast<const float4 *>(lv), p1 = *reinterpret_cast<const float4 *>(lv + 4);
             if (dn & 1) o0.x = p0.x;

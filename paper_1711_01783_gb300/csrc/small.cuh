@@ -137,7 +137,7 @@ __device__ __forceinline__ void small_check(const CnArgs &a, const ClassLaunch &
     t.pp = a.phi1 + (static_cast<size_t>(slab) * a.n_deg1 + s0) * W + lane0;
     const uint32_t sb =
         static_cast<uint32_t>(a.sbits[(static_cast<size_t>(slab) * a.n_cn + cl.c0 + j) * NB + lane0 / 8]) >> (lane0 & 7);
-    const uint32_t donenib = a.et ? stopped_nibble<W>(a, slab, lane0) : 0u;
+    const uint32_t donenib = a.et ? kept_nibble<W, PASS == kPassFull>(a, slab, lane0) : 0u;
     check_terms<MsgT, W, DC, DD, PASS, false, false>(a, lane0, slab, true, rp, e0, s0, sb, donenib, t);
 }
 
@@ -281,9 +281,10 @@ bool launch_small(mld_decoder *d, int32_t batch, int32_t iters, bool et, bool ha
     s.status = d->status;
     s.stall = d->stall_test;
     s.cn = CnArgs{g->cptr, g->col, g->dptr, h.n_cn, h.n_core, h.n_deg1, h.e_core, d->r, d->Lv, d->lch1, d->phi1,
-                  d->post1, d->hb1, d->sbits, nullptr, d->lmax_i, d->amin_i, 0, et ? 1 : 0, batch};
+                  d->post1, d->hb1, d->sbits, nullptr, d->lmax_i, d->amin_i, 0, et ? 1 : 0};
+    s.cn.batch = batch;
     if (!et && !soft) s.cn.post1 = nullptr;
-    s.vn = VnArgs{g->vptr, g->vedge, h.n_core, h.e_core, d->r, d->lch, d->Lv, d->hb_core, nullptr, 0, et ? 1 : 0, batch};
+    s.vn = VnArgs{g->vptr, g->vedge, h.n_core, h.e_core, d->r, d->lch, d->Lv, d->hb_core, nullptr, 0, et ? 1 : 0};
     s.sy = SynArgs{g->cptr, g->col, g->dptr, h.n_cn, h.n_core, h.n_deg1, d->sbits, d->hb_core, d->hb1, d->fail,
                    nullptr, et ? 1 : 0, batch};
     if (launches.empty() || launches.size() > kSmallMaxClasses || s.batch > kSmallMaxLanes) return false;
