@@ -385,8 +385,9 @@ int mld_decoder_test_stall(mld_decoder *d, int32_t bytes);
  * Semantics per codeword are those of mld_decode_y / mld_decode with the
  * job's max_iters; with MLD_EARLY_TERM each codeword stops at its first
  * syndrome match (Methods, Step 5) and a slab whose codewords have all
- * stopped is skipped; the iterations are then a loop inside the graph, which
- * the device leaves once every codeword has stopped.
+ * stopped is skipped; the iterations are then a loop inside the graph, or a few
+ * where the jobs that are past their caps outweigh the others, which the device
+ * leaves once every codeword has stopped.
  *   decoder    : from mld_decoder_create; at most one job per decoder.
  *   in         : device float [batch][n_vn]: observations y if sigma != NULL
  *                (LLR = 2y/sigma^2 formed on the device), else channel LLRs.
@@ -415,11 +416,16 @@ typedef struct {
 } mld_job;
 typedef struct mld_plan mld_plan;
 int mld_plan_create(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan **out);
-/* Enqueue the plan's CUDA graph on `stream` (one launch). */
+/* Enqueue the plan's CUDA graph on `stream` (one launch).  Not on a stream that
+ * is being captured: CUDA does not capture the launch of a graph (MLD_ECUDA). */
 int mld_plan_launch(mld_plan *p, void *stream);
 /* Number of kernel launches inside the plan's graph (with early termination
- * the loop's body, two iterations, counts once). */
+ * the body of each loop, two iterations, counts once). */
 int mld_plan_stats(const mld_plan *p, int64_t *launches);
+/* Number of kernels that a launch of the plan runs when its last codeword stops
+ * at iteration `iterations` (the largest iters_used of its jobs; without early
+ * termination it makes no difference). */
+int mld_plan_launched(const mld_plan *p, int32_t iterations, int64_t *launches);
 int mld_plan_destroy(mld_plan *p);
 /* Create a plan, launch it on `stream`, wait for the stream, destroy it. */
 int mld_decode_multi(const mld_job *jobs, int32_t n_jobs, uint32_t flags, void *stream);

@@ -41,7 +41,7 @@ _STATUS = {MLD_EINVAL: "MLD_EINVAL", MLD_ENOMEM: "MLD_ENOMEM", MLD_ECUDA: "MLD_E
 EXPORTS = ("mld_last_error", "mld_version", "mld_graph_create", "mld_graph_destroy",
            "mld_graph_stats_get", "mld_decoder_create", "mld_decoder_destroy", "mld_decode",
            "mld_decode_y", "mld_decode_status", "mld_decoder_one_launch", "mld_decoder_test_stall", "mld_decoder_timing_enable",
-           "mld_decoder_timing_read", "mld_decode_noalloc", "mld_plan_create", "mld_plan_launch",
+           "mld_decoder_timing_read", "mld_decode_noalloc", "mld_plan_create", "mld_plan_launch", "mld_plan_launched",
            "mld_plan_stats", "mld_plan_destroy", "mld_decode_multi", "mld_wbp_forward", "mld_wbp_backward",
            "mld_tape_destroy", "mld_phi_eval", "mld_ensemble_size", "mld_ensemble_edges",
            "mld_graph_generate", "mld_graph_set_layers", "mld_graph_layers_get", "mld_md_bob", "mld_md_alice", "mld_peg_edges", "mld_graph_index_arrays")
@@ -121,6 +121,7 @@ def _load() -> ctypes.CDLL:
         "mld_plan_create": (ctypes.c_int, [P, I32, U32, ctypes.POINTER(P)]),
         "mld_plan_launch": (ctypes.c_int, [P, P]),
         "mld_plan_stats": (ctypes.c_int, [P, ctypes.POINTER(I64)]),
+        "mld_plan_launched": (ctypes.c_int, [P, I32, ctypes.POINTER(I64)]),
         "mld_plan_destroy": (ctypes.c_int, [P]),
         "mld_decode_multi": (ctypes.c_int, [P, I32, U32, P]),
         "mld_wbp_forward": (ctypes.c_int, [P, P, P, I32, P, I32, I32, I32, P, ctypes.POINTER(P), P]),
@@ -551,6 +552,13 @@ class Plan:
         n = ctypes.c_int64()
         _check(lib().mld_plan_stats(h, ctypes.byref(n)))
         self.launches = int(n.value)
+
+    def launched(self, iterations: int) -> int:
+        """Kernels that a launch runs when its last codeword stops at iteration
+        ``iterations`` (mld_plan_launched)."""
+        n = ctypes.c_int64()
+        _check(lib().mld_plan_launched(self._h, int(iterations), ctypes.byref(n)))
+        return int(n.value)
 
     def launch(self, stream=None):
         _check(lib().mld_plan_launch(self._h, _stream_handle(stream)))

@@ -1,8 +1,8 @@
 // Uneven batches: many codewords over several Tanner graphs (different
 // rates and lengths), each group with its own iteration cap, decoded by one
 // schedule of launches that is captured once into a CUDA graph and replayed
-// with a single launch.  With early termination the iterations are the body of
-// a conditional loop inside that graph, run by the device until every codeword
+// with a single launch.  With early termination the iterations are the bodies of
+// conditional loops inside that graph, run by the device until every codeword
 // has stopped.
 //
 // The paper decodes a batch of codewords of one code with a fixed number of
@@ -14,6 +14,7 @@
 // syndrome match or at its job's cap; its slab is skipped once all its
 // codewords have stopped, and lanes past the batch count as stopped from the
 // start.
+#include <algorithm>
 #include <map>
 #include <tuple>
 #include <type_traits>
@@ -174,21 +175,33 @@ __global__ void __launch_bounds__(kBlock) km_init(const JobDev *jobs, int32_t *l
     if (blockIdx.x == 0 && threadIdx.x == 0) *lctr = 0;
 }
 
-// Continue while some lane of some job still iterates, counting the body's two
-// iterations (one block).
-__global__ void __launch_bounds__(kBlock) km_loop_cond(const JobDev *jobs, int n_jobs, int32_t *lctr,
-                                                       cudaGraphConditionalHandle h) {
+// Whether every lane of every job has stopped (one block).
+__device__ __forceinline__ bool all_stopped(const JobDev *jobs, int n_jobs) {
     bool all = true;
     for (int k = 0; k < n_jobs; ++k) {
         const JobDev &j = jobs[k];
         const uint32_t full = j.W >= 32 ? 0xFFFFFFFFu : ((1u << j.W) - 1u);
         for (int i = threadIdx.x; i < j.slabs * ((j.W + 31) / 32); i += blockDim.x) all = all && j.done[i] == full;
     }
-    all = __syncthreads_and(all);
+    return __syncthreads_and(all) != 0;
+}
+
+// End of a loop's body: counts its two iterations; continue while some lane
+// still iterates and fewer than `end` are done.
+__global__ void __launch_bounds__(kBlock) km_loop_cond(const JobDev *jobs, int n_jobs, int32_t *lctr, int32_t end,
+                                                       cudaGraphConditionalHandle h) {
+    const bool all = all_stopped(jobs, n_jobs);
     if (threadIdx.x == 0) {
-        if (!all) *lctr += 2;
-        cudaGraphSetConditional(h, all ? 0u : 1u);
+        const int32_t l = *lctr + (all ? 0 : 2);
+        *lctr = l;
+        cudaGraphSetConditional(h, !all && l < end ? 1u : 0u);
     }
+}
+
+// Before a later loop: enter it if some lane still iterates.
+__global__ void __launch_bounds__(kBlock) km_loop_enter(const JobDev *jobs, int n_jobs, cudaGraphConditionalHandle h) {
+    const bool all = all_stopped(jobs, n_jobs);
+    if (threadIdx.x == 0) cudaGraphSetConditional(h, all ? 0u : 1u);
 }
 
 template <int W, int F>
@@ -239,11 +252,16 @@ struct mld_plan {
     int device = 0;
     JobDev *d_jobs = nullptr;
     Seg *d_segs = nullptr;
-    int32_t *d_lctr = nullptr;  // iterations before the loop's current body
+    int32_t *d_lctr = nullptr;  // iterations before the current loop body
     int n_jobs = 0;
-    // the schedule: before, one body of the early-termination loop (empty
-    // without one), after
-    std::vector<Op> before, body, after;
+    // the schedule: before, the early-termination loops (none without early
+    // termination), after
+    struct Loop {
+        std::vector<Op> body;  // two iterations
+        int32_t end;           // left when so many iterations are done
+    };
+    std::vector<Op> before, after;
+    std::vector<Loop> loops;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -344,8 +362,8 @@ int capture_into(cudaGraph_t g, cudaStream_t cs, F &&fill) {
     return MLD_OK;
 }
 
-// The plan's graph: the ops before the loop, the loop (a conditional node
-// whose body graph holds two iterations), the ops after it.
+// The plan's graph: the ops before the loops, the loops (conditional nodes
+// whose body graphs hold two iterations), the ops after them.
 int build_graph(mld_plan *p, cudaStream_t cs) {
     MLD_CUDA(cudaGraphCreate(&p->graph, 0));
     cudaGraphNode_t last = nullptr;
@@ -365,9 +383,21 @@ int build_graph(mld_plan *p, cudaStream_t cs) {
     };
     int s = add_ops(p->before);
     if (s != MLD_OK) return s;
-    if (!p->body.empty()) {
+    for (size_t k = 0; k < p->loops.size(); ++k) {
+        const mld_plan::Loop &loop = p->loops[k];
         cudaGraphConditionalHandle h;
         MLD_CUDA(cudaGraphConditionalHandleCreate(&h, p->graph, 1, cudaGraphCondAssignDefault));
+        if (k > 0) {
+            void *args[] = {&p->d_jobs, &p->n_jobs, &h};
+            cudaKernelNodeParams kp{};
+            kp.func = reinterpret_cast<void *>(&km_loop_enter);
+            kp.gridDim = dim3(1);
+            kp.blockDim = dim3(kBlock);
+            kp.kernelParams = args;
+            cudaGraphNode_t enter = nullptr;
+            MLD_CUDA(cudaGraphAddKernelNode(&enter, p->graph, &last, 1, &kp));
+            last = enter;
+        }
         cudaGraphNodeParams np{};
         np.type = cudaGraphNodeTypeConditional;
         np.conditional.handle = h;
@@ -377,15 +407,21 @@ int build_graph(mld_plan *p, cudaStream_t cs) {
         MLD_CUDA(cudaGraphAddNode(&node, p->graph, &last, nullptr, 1, &np));
         last = node;
         s = capture_into(np.conditional.phGraph_out[0], cs, [&](cudaStream_t st) -> int {
-            const int q = enqueue(p, p->body, st);
+            const int q = enqueue(p, loop.body, st);
             if (q != MLD_OK) return q;
-            km_loop_cond<<<1, kBlock, 0, st>>>(p->d_jobs, p->n_jobs, p->d_lctr, h);
+            km_loop_cond<<<1, kBlock, 0, st>>>(p->d_jobs, p->n_jobs, p->d_lctr, loop.end, h);
             MLD_LAUNCHED("km_loop_cond");
             return MLD_OK;
         });
         if (s != MLD_OK) return s;
     }
     return add_ops(p->after);
+}
+
+int64_t kernels(const std::vector<Op> &ops) {
+    int64_t n = 0;
+    for (const Op &op : ops) n += (op.kind == kOpMemset) ? 0 : 1;
+    return n;
 }
 
 void plan_free(mld_plan *p) {
@@ -590,15 +626,43 @@ int build_plan(const mld_job *jobs, int32_t n_jobs, uint32_t flags, mld_plan *p,
         if (!checked.empty()) syndrome_round(checked, l);
     };
     if (et) {
-        // the device repeats two iterations until every codeword has stopped
-        std::vector<int32_t> active;
-        for (int32_t j = 0; j < n_jobs; ++j)
-            if (jobs[j].max_iters > 0) active.push_back(j);
-        if (!active.empty()) {
-            ops = &p->body;
+        // the device repeats two iterations until every codeword has stopped.  A
+        // job past its cap still launches blocks that find nothing to do, so a
+        // new loop without them begins where they outnumber the blocks of the
+        // jobs that go on four to one (64 codewords of n = 200000 with a cap of 2
+        // beside three of n = 4096 with one of 200: 6.0 ms in one loop, 3.9 ms in
+        // two); not sooner, since a further loop costs 0.15 ms and more a launch
+        // (96 codewords in nine jobs of three caps, all stopped at the first:
+        // 15.2 ms in one loop, 15.5 ms in two or three)
+        std::vector<std::pair<int32_t, int64_t>> caps;  // rounded up to even, blocks of an iteration
+        int64_t going_on = 0, past = 0;
+        for (int32_t j = 0; j < n_jobs; ++j) {
+            if (jobs[j].max_iters == 0) continue;
+            const mld::HostGraph &h = jobs[j].decoder->g->h;
+            int64_t b = grid_x(static_cast<int64_t>(h.n_core) * (jd[j].W / kVnLanes)) + syndrome_blocks(jd[j].n_cn, sm_count);
+            for (const ClassLaunch &cl : jobs[j].decoder->g->launches[width_index(jd[j].W)])
+                b += cl.dc >= 0 ? class_blocks(cl, sm_count) : cl.blocks;
+            b *= jd[j].slabs;
+            caps.push_back({static_cast<int32_t>(std::min<int64_t>((jobs[j].max_iters + 1LL) / 2 * 2, INT32_MAX)), b});
+            going_on += b;
+        }
+        std::sort(caps.begin(), caps.end());
+        int32_t begin = 0;
+        for (size_t k = 0; k < caps.size(); ++k) {
+            past += caps[k].second;
+            going_on -= caps[k].second;
+            const bool last = k + 1 == caps.size();
+            if (!last && (caps[k + 1].first == caps[k].first || past <= 4 * going_on)) continue;
+            std::vector<int32_t> active;
+            for (int32_t j = 0; j < n_jobs; ++j)
+                if (jobs[j].max_iters > begin) active.push_back(j);
+            p->loops.push_back({{}, caps[k].first});
+            ops = &p->loops.back().body;
             in_loop = true;
             for (int32_t l = 1; l <= 2; ++l) iteration(active, l, [](int32_t) { return true; });
             in_loop = false;
+            begin = caps[k].first;
+            past = 0;
         }
     } else {
         for (int32_t l = 1; l <= lmax_iters; ++l) {
@@ -694,9 +758,21 @@ int mld_plan_stats(const mld_plan *p, int64_t *launches) {
     mld::clear_error();
     if (!p || !launches) return mld::fail(MLD_EINVAL, "plan_stats: null pointer");
     int64_t n = 0;
-    for (const std::vector<Op> *part : {&p->before, &p->body, &p->after})
-        for (const Op &op : *part) n += (op.kind == kOpMemset) ? 0 : 1;
-    if (!p->body.empty()) n += 1;  // the loop's condition
+    for (size_t k = 0; k < p->loops.size(); ++k) n += kernels(p->loops[k].body) + (k > 0 ? 2 : 1);  // and its conditions
+    *launches = n + kernels(p->before) + kernels(p->after);
+    return MLD_OK;
+}
+
+int mld_plan_launched(const mld_plan *p, int32_t iterations, int64_t *launches) {
+    mld::clear_error();
+    if (!p || !launches) return mld::fail(MLD_EINVAL, "plan_launched: null pointer");
+    if (iterations < 0) return mld::fail(MLD_EINVAL, "plan_launched: negative iterations");
+    int64_t n = kernels(p->before) + kernels(p->after), l = 0;
+    for (size_t k = 0; k < p->loops.size(); ++k) {
+        if (k > 0) n += 1;  // its entry condition
+        for (bool first = k == 0; first || (l < iterations && l < p->loops[k].end); first = false, l += 2)
+            n += kernels(p->loops[k].body) + 1;
+    }
     *launches = n;
     return MLD_OK;
 }
