@@ -3,18 +3,20 @@
 The slab width W (codewords interleaved per 128-byte line group: 8, 16, 32
 or 64) trades padding against access granularity: a batch of 11 codewords
 fills 69 % of a 16-wide slab but 17 % of a 64-wide one, while wider slabs
-move whole 128-byte lines per graph access.  The tuner times a few decoder
-iterations for every width on the actual graph and batch size, keeps the
+move whole 128-byte lines per graph access.  The tuner times a few iterations
+of a one-job plan for every width on the actual graph and batch size, keeps the
 fastest per decoded codeword, and caches the choice in a JSON file keyed by
-(graph signature, batch, message type, GPU name).
+(graph signature, batch, message type, GPU name).  It times a plan because a
+plan is what the width is for: a decode call of a small problem runs in one
+launch, whose best width is another.
 
 ``DecoderTuner`` widens the search for single-graph decoding without early
 termination to the variable-update variant as well: the gather pass or the
 accumulation of the new messages inside the check update (which wins with
 float messages and loses with half ones on GB300), over the slab widths each
 variant allows, and for half messages to the staged check update (operands
-brought into shared memory by block-wide bulk copies; slower on GB300).  Plans keep the gather, so they use
-``SlabWidthTuner``.
+brought into shared memory by block-wide bulk copies; slower on GB300).  It
+times decode calls.  Plans keep the gather, so they use ``SlabWidthTuner``.
 """
 from __future__ import annotations
 
@@ -37,12 +39,12 @@ class SlabWidthTuner:
 
     def _key(self, graph, batch: int, msg_dtype: str) -> str:
         import torch
-        return f"{graph.signature}|{batch}|{msg_dtype}|{torch.cuda.get_device_name()}"
+        return f"plan|{graph.signature}|{batch}|{msg_dtype}|{torch.cuda.get_device_name()}"
 
     def choose(self, graph, batch: int, msg_dtype: str = "f16") -> int:
         import torch
 
-        from . import Decoder
+        from . import Decoder, Plan
         key = self._key(graph, batch, msg_dtype)
         if key in self.cache:
             return int(self.cache[key]["W"])
@@ -52,15 +54,17 @@ class SlabWidthTuner:
         times = {}
         for W in WIDTHS:
             dec = Decoder(graph, batch, msg_dtype=msg_dtype, slab_width=W)
-            dec.decode(llr, syn, self.iters)
+            plan = Plan([dict(decoder=dec, y=llr, syndrome=syn, max_iters=self.iters)])
+            plan.launch()
             torch.cuda.synchronize()
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             e0.record()
             for _ in range(self.reps):
-                dec.decode(llr, syn, self.iters)
+                plan.launch()
             e1.record()
             torch.cuda.synchronize()
             times[W] = e0.elapsed_time(e1) / self.reps
+            plan.close()
             dec.close()
         best = min(times, key=times.get)
         self.cache[key] = {"W": best, "ms": times}
@@ -78,7 +82,7 @@ class DecoderTuner(SlabWidthTuner):
     batch; cached like the slab width."""
 
     def _key(self, graph, batch: int, msg_dtype: str) -> str:
-        return "dec|" + super()._key(graph, batch, msg_dtype)
+        return "dec|" + super()._key(graph, batch, msg_dtype).removeprefix("plan|")
 
     def candidates(self, msg_dtype: str):
         default_w = 64 if msg_dtype == "f16" else 32
