@@ -79,13 +79,13 @@ DEFAULT_ITERS = {0.1: 100, 0.05: 150, 0.02: 200}
 # the launching stream); sampling keeps the event records out of the step time.
 TIMING_EVERY = 10
 
-# DRAM bytes (read + write) of one check-update pass per (codeword x bit),
-# from ncu's dram__bytes_read.sum + dram__bytes_write.sum of the three
-# check-class launches of one iteration (rate 0.1, n = 3e5, 64 codewords,
-# half messages: 395.94 MB); traffic grows with n, so it is scaled by the
-# units a full pass processes.  Valid for the kernel of this commit only
-# (see profiles/).
-CHECK_PASS_TRAFFIC_PER_CW_BIT = {(0.1, "f16"): 395.94e6 / (64 * 3e5)}
+# DRAM bytes (read + write) of one check-update pass, ncu's
+# dram__bytes_read.sum + dram__bytes_write.sum of the three check-class launches
+# of one iteration, by (rate, message type, n, codewords).  Only sizes that were
+# measured: the traffic does not grow in proportion to n (at n = 10^6 the
+# posteriors no longer stay in L2 between the passes).  Valid for the kernel of
+# this commit only (see profiles/).
+CHECK_PASS_TRAFFIC = {(0.1, "f16", 300_000, 64): 395.94e6, (0.1, "f16", 1_000_000, 64): 1.57e9}
 
 
 def algorithmic_bytes(st: dict, msg: str, schedule: str = "flooding") -> tuple[float, float]:
@@ -304,7 +304,8 @@ def uneven_record(total: int, beta: float, msg: str, steps: int, warmup: int, ra
     rec = {"value": bits / (ms * 1e-3) / 1e6, "unit": UNIT, "ms_per_step": ms, "steps": steps, "warmup": warmup,
            "workload": f"{total} codewords, (rate, n) uniform over {{0.1,0.05,0.02}} x {{2^16,2^18,10^6}}, "
                        f"caps 100/150/200, early termination, beta={beta}, {msg} messages",
-           "groups (batch, slab width)": widths, "gpu_launches": plan.launches * steps,
+           "groups (batch, slab width)": widths,
+           "gpu_launches": plan.launched(max(int(o["iters_used"].max().item()) for o in outs)) * steps,
            "frames_converged": sum(int(o["converged"].sum().item()) for o in outs),
            "mean_iters": [round(float(o["iters_used"].float().mean().item()), 2) for o in outs]}
     plan.close()
@@ -791,9 +792,9 @@ def main():
     peak, peak_kind = measured_peak_hbm()
     ks = kernel_summary(kt, st, a.msg, a.batch, a.iters, a.steps, ms_max / a.steps, peak)
     # the counters were taken on the gather variant's check kernel
-    tpb = CHECK_PASS_TRAFFIC_PER_CW_BIT.get((a.rate, a.msg)) if a.vn_update == "gather" else None
+    traffic = CHECK_PASS_TRAFFIC.get((a.rate, a.msg, a.n, a.batch)) if a.vn_update == "gather" else None
     roofline = {"bound": "hbm", "achieved": ks["achieved"], "peak": peak, "unit": "GB/s",
-                "frac": ks["frac"], "traffic": tpb * a.batch * a.n if tpb else None,
+                "frac": ks["frac"], "traffic": traffic,
                 "kernel": "k_check_update (one pass = all check classes of one iteration)",
                 "peak_kind": peak_kind}
     roofline.update({k: v for k, v in ks.items() if k not in ("achieved", "frac")})

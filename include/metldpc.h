@@ -329,7 +329,10 @@ int mld_decoder_destroy(mld_decoder *d);
  * wait on one another at most 2 s.  Should such a wait run out, the decode
  * gives up: converged and iters_used are 0 for every codeword, bits and
  * posteriors are unfinished, and mld_decode_status returns MLD_ETIMEOUT from
- * then on (later decodes of this kind on that decoder give up at once). */
+ * then on (later decodes of this kind on that decoder give up at once).  Such
+ * a decode keeps its SMs to itself until it ends, half of them or all: decodes
+ * on several streams at once share the GPU by turns.  One batch, or one plan,
+ * decodes them together. */
 int mld_decode(mld_decoder *d, const float *llr, const uint8_t *syndrome,
                int32_t batch, int32_t max_iters, uint32_t flags,
                uint8_t *bits_out, float *post_out, uint8_t *converged,
@@ -484,7 +487,10 @@ int mld_tape_destroy(mld_tape *t);
  * while timing was on (*_launches, sampled or not); then it clears them.
  * Classes: check update (Eqs. 2-3), variable update (Eqs. 4-5), syndrome
  * check (Step 5), layout (interleave / de-interleave / bit packing).
- * Timing changes no result.  Errors: MLD_EINVAL, MLD_ECUDA. */
+ * Timing changes no result, but a small problem's decode leaves its one launch
+ * (see mld_decode) for a launch per class and phase while it is on: what is
+ * timed is then not the kernel that runs otherwise.  Errors: MLD_EINVAL,
+ * MLD_ECUDA. */
 typedef struct {
     double check_ms, var_ms, syndrome_ms, layout_ms;
     int64_t check_launches, var_launches, syndrome_launches, layout_launches;
