@@ -85,7 +85,7 @@ TIMING_EVERY = 10
 # measured: the traffic does not grow in proportion to n (at n = 10^6 the
 # posteriors no longer stay in L2 between the passes).  Valid for the kernel of
 # this commit only (see profiles/).
-CHECK_PASS_TRAFFIC = {(0.1, "f16", 300_000, 64): 395.94e6, (0.1, "f16", 1_000_000, 64): 1.57e9}
+CHECK_PASS_TRAFFIC = {(0.1, "f16", 300_000, 64): 395.94e6, (0.1, "f16", 1_000_000, 64): 1.75e9}
 
 
 def algorithmic_bytes(st: dict, msg: str, schedule: str = "flooding") -> tuple[float, float]:
